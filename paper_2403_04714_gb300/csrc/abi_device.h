@@ -98,9 +98,11 @@ constexpr uint32_t kNoProc = 0xffffffffu;
 
 // State of one batch of instances (device pointers).
 struct DevState {
-    uint32_t* bits[2];          // 1-bit registers: [n_bit][bit_stride] words, `pack` instances per word
-    uint32_t* w32[2];           // 2..32-bit registers: [n_w32][I]
-    uint64_t* w64[2];           // 33..64-bit registers: [n_w64][I]
+    // registers; with lane = instance (pack 32) in tiles of one instance group:
+    // [group][register][32 instances], one word of 32 instances per 1-bit register
+    uint32_t* bits[2];          // 1-bit registers: [n_bit][I] words, or [I / 32][n_bit]
+    uint32_t* w32[2];           // 2..32-bit registers: [n_w32][I], or [I / 32][n_w32][32]
+    uint64_t* w64[2];           // 33..64-bit registers: [n_w64][I], or [I / 32][n_w64][32]
     uint64_t* mem;              // all memories, instance-minor
     uint64_t* rec[2];           // write records [n_wport][I][2]: (en<<63 | addr, data)
     const uint64_t* key;        // stimulus key per instance
@@ -113,10 +115,11 @@ struct DevState {
     const uint64_t* rom_dig;    // digest of the memories without write ports, per instance
     uint32_t* bar;              // grid barrier words: [0] arrivals, [1] generation
     int32_t* err;               // first error code of the launch (0 = none)
-    uint64_t* stim[2];          // generated code: input k of instance i at cycle t in stim[t & 1][k * I + i], or null
+    uint64_t* stim[2];          // generated code: input k of instance i at cycle t in stim[t & 1][(i / 32 * n_in + k) * 32 + i % 32]
+                                // (one instance per warp: [k * I + i]), or null
     uint32_t I;                 // instances (padded to the lane-group size)
     uint32_t pack;              // instances per bit word (32 LANE_INST, 1 LANE_OP)
-    uint32_t bit_stride;        // words per 1-bit register
+    uint32_t n_bit, n_w32, n_w64;   // registers of each class
     uint32_t any_hold;          // some input is held
     uint32_t ring_cap;          // 0 = digests off
     uint32_t n_tracked;

@@ -61,6 +61,11 @@ struct Emitter {
         if (d.op == OP_CONST) return d.w <= 32 ? std::to_string(uint32_t(d.k)) + "u" : hex64(d.k);
         return "v" + std::to_string(local[n]);
     }
+    // position of register (or input) ix in its plane, after the group's base
+    std::string pos(uint32_t ix) const {
+        if (mode != SIM_MODE_LANE_INST) return std::to_string(ix) + "ull * I + inst";
+        return std::to_string(uint64_t(ix) * 32) + "u";
+    }
     std::string ref64(int32_t n) const { return "((uint64_t)" + ref(n) + ")"; }
     bool wide(int32_t n) const { return nl.nodes[n].w > 32; }
 
@@ -74,14 +79,14 @@ struct Emitter {
         switch (d.op) {
         case OP_REG: {
             const uint32_t ix = L.idx[d.a];
-            if (L.cls[d.a] == RC_W64) e = "c64[" + std::to_string(ix) + "ull * I + inst]";
-            else if (L.cls[d.a] == RC_W32) e = "c32[" + std::to_string(ix) + "ull * I + inst]";
-            else if (mode == SIM_MODE_LANE_INST) e = "(c1[" + std::to_string(ix) + "ull * BS + g] >> lane) & 1u";
-            else e = "c1[" + std::to_string(ix) + "ull * BS + inst]";
+            if (L.cls[d.a] == RC_W64) e = "c64[" + pos(ix) + "]";
+            else if (L.cls[d.a] == RC_W32) e = "c32[" + pos(ix) + "]";
+            else if (mode == SIM_MODE_LANE_INST) e = "(c1[" + std::to_string(ix) + "u] >> lane) & 1u";
+            else e = "c1[" + std::to_string(ix) + "ull * I + inst]";
             break;
         }
         case OP_INPUT:      // the value filled for this cycle (already reduced to the input's width)
-            e = "(" + T + ")stv[" + std::to_string(d.a) + "ull * I + inst]";
+            e = "(" + T + ")stv[" + pos(uint32_t(d.a)) + "]";
             break;
         case OP_MEMRD:
             e = "(" + T + ")mem_read(P, S, " + std::to_string(d.a) + "u, " + ref64(d.b) + " & " +
@@ -151,14 +156,14 @@ struct Emitter {
         const uint32_t ix = L.idx[r];
         o += "    { const uint64_t sv = " + val + ";\n";
         if (L.cls[r] == RC_W64) {
-            o += "      n64[" + std::to_string(ix) + "ull * I + inst] = sv;\n";
+            o += "      n64[" + pos(ix) + "] = sv;\n";
         } else if (L.cls[r] == RC_W32) {
-            o += "      n32[" + std::to_string(ix) + "ull * I + inst] = (uint32_t)sv;\n";
+            o += "      n32[" + pos(ix) + "] = (uint32_t)sv;\n";
         } else if (mode == SIM_MODE_LANE_INST) {
             o += "      const uint32_t wb = __ballot_sync(0xffffffffu, (sv & 1u) != 0);\n"
-                 "      if (lane == 0) n1[" + std::to_string(ix) + "ull * BS + g] = wb;\n";
+                 "      if (lane == 0) n1[" + std::to_string(ix) + "u] = wb;\n";
         } else {
-            o += "      n1[" + std::to_string(ix) + "ull * BS + inst] = (uint32_t)sv;\n";
+            o += "      n1[" + std::to_string(ix) + "ull * I + inst] = (uint32_t)sv;\n";
         }
         if (digest)
             o += "      if (col >= 0) *dacc += mix64((" + hex64(uint64_t(r) * 0x9E3779B97F4A7C15ULL + 1ULL) + ") ^ sv);\n";
@@ -267,13 +272,20 @@ void gen_process(const Netlist& nl, const Partition& part, const RegLayout& L, s
          "    using namespace rtl;\n"
          "    const DevProg& P = *Pp;\n    const DevState& S = *Sp;\n"
          "    const uint32_t par = (uint32_t)(t & 1), nxt = par ^ 1u;\n"
-         "    const uint64_t I = S.I, BS = S.bit_stride;\n";
+         "    const uint64_t I = S.I;\n    (void)I;\n";
     o += mode == SIM_MODE_LANE_INST ? "    const uint32_t inst = g * 32u + lane;\n" : "    const uint32_t inst = g;\n";
-    o += "    const uint64_t* __restrict__ c64 = S.w64[par];\n    uint64_t* __restrict__ n64 = S.w64[nxt];\n"
-         "    const uint32_t* __restrict__ c32 = S.w32[par];\n    uint32_t* __restrict__ n32 = S.w32[nxt];\n"
-         "    const uint32_t* __restrict__ c1 = S.bits[par];\n    uint32_t* __restrict__ n1 = S.bits[nxt];\n"
-         "    (void)c64; (void)n64; (void)c32; (void)n32; (void)c1; (void)n1; (void)BS; (void)lane; (void)pending;\n";
-    if (has_input) o += "    const uint64_t* __restrict__ stv = S.stim[par];\n";
+    // lane = instance: the group's tile (reg_pos), every register a constant offset from it
+    auto base = [&](uint32_t n, bool words) {
+        if (mode != SIM_MODE_LANE_INST) return std::string();
+        return words ? " + (uint64_t)g * " + std::to_string(n) + "u"
+                     : " + ((uint64_t)g * " + std::to_string(n) + "u * 32u + lane)";
+    };
+    const std::string b64 = base(L.count[RC_W64], false), b32 = base(L.count[RC_W32], false), b1 = base(L.count[RC_BIT], true);
+    o += "    const uint64_t* __restrict__ c64 = S.w64[par]" + b64 + ";\n    uint64_t* __restrict__ n64 = S.w64[nxt]" + b64 + ";\n"
+         "    const uint32_t* __restrict__ c32 = S.w32[par]" + b32 + ";\n    uint32_t* __restrict__ n32 = S.w32[nxt]" + b32 + ";\n"
+         "    const uint32_t* __restrict__ c1 = S.bits[par]" + b1 + ";\n    uint32_t* __restrict__ n1 = S.bits[nxt]" + b1 + ";\n"
+         "    (void)c64; (void)n64; (void)c32; (void)n32; (void)c1; (void)n1; (void)lane; (void)pending;\n";
+    if (has_input) o += "    const uint64_t* __restrict__ stv = S.stim[par]" + base(uint32_t(nl.in_w.size()), false) + ";\n";
     for (int32_t f : part.procs[p])
         if (part.fibers[f].mem >= 0) E.commit(part.fibers[f].mem);
     for (int32_t f : fiber_order(part, p, E.local, nodes.size())) {

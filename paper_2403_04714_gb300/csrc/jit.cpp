@@ -57,13 +57,13 @@ void write_file(const std::string& path, const std::vector<char>& data) {
 
 // Registers per thread for generated code.  Process functions with many live
 // values would otherwise claim up to 255 registers and hold one 256-thread
-// CTA per SM.  Measured on the 200k-op netlist with 4,096 instances (8-warp
-// CTAs): uncapped 3.6M instance-cycles/s; 64 registers (4 CTAs per SM) 6.9M;
-// 80 (3 CTAs) 7.5M; 96 and 128 (2 CTAs) 4.8-5.0M.  Spills fall from 1.9 GB
-// to 1.3 GB of local traffic per simulated cycle between 64 and 80.
+// CTA per SM.  Measured on the 200k-op netlist with 4,096 instances (us per
+// simulated cycle, best CTA size): 48 registers 198, 56 204, 64 186, 72 197,
+// 80 203, 96 216.  At 64 the state's constant offsets (reg_pos) leave few
+// spills (27 local loads per task) and 32 warps share an SM.
 std::string max_registers() {
     const char* m = getenv("RTLSIM_GEN_MAXRREG");
-    return m ? m : "80";
+    return m ? m : "64";
 }
 
 // The kernel entry's launch bound must leave every process function its

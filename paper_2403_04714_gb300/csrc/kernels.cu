@@ -108,12 +108,12 @@ __device__ void task_lane_inst(const DevProg& P, const DevState& S, uint32_t p, 
             uint64_t v = SL(d.a) & wmask(d.w);
             uint32_t idx = d.b | (d.x << 16);
             if (d.c == RC_W64) {
-                S.w64[nxt][(uint64_t)idx * S.I + inst] = v;
+                S.w64[nxt][reg_pos(S, S.n_w64, idx, inst)] = v;
             } else if (d.c == RC_W32) {
-                S.w32[nxt][(uint64_t)idx * S.I + inst] = uint32_t(v);
+                S.w32[nxt][reg_pos(S, S.n_w32, idx, inst)] = uint32_t(v);
             } else {
                 uint32_t word = __ballot_sync(0xffffffffu, v & 1);
-                if (lane == 0) S.bits[nxt][(uint64_t)idx * S.bit_stride + g] = word;
+                if (lane == 0) S.bits[nxt][(uint64_t)g * S.n_bit + idx] = word;
             }
             if (DIGEST && col >= 0) dacc += mix64(((uint64_t)d.imm * kGamma + 1ULL) ^ v);
             break;
@@ -266,7 +266,7 @@ __device__ __forceinline__ void store_reg(const Dec& d, uint64_t v, const DevSta
     const uint32_t idx = d.b | (d.x << 16);
     if (d.c == RC_W64) S.w64[nxt][(uint64_t)idx * S.I + inst] = v;
     else if (d.c == RC_W32) S.w32[nxt][(uint64_t)idx * S.I + inst] = uint32_t(v);
-    else S.bits[nxt][(uint64_t)idx * S.bit_stride + inst] = uint32_t(v);
+    else S.bits[nxt][(uint64_t)idx * S.I + inst] = uint32_t(v);
     if (DIGEST && col >= 0) dacc += mix64(((uint64_t)d.imm * kGamma + 1ULL) ^ v);
 }
 
@@ -284,7 +284,7 @@ __device__ __forceinline__ void exec_lane_op(const Dec& d, const DevProg& P, con
     case D_NOP:
         break;
     case D_LDR:
-        sl[d.dst] = load_reg(S, par, d.c, d.b | (d.x << 16), inst);
+        sl[d.dst] = load_reg1(S, par, d.c, d.b | (d.x << 16), inst);
         break;
     case D_LDI:
         sl[d.dst] = stimulus(P, S, key, d.imm, inst, t, d.w);
@@ -329,7 +329,7 @@ __device__ __forceinline__ void exec_lane_op(const Dec& d, const DevProg& P, con
 // Value of a leaf instruction (register, mirror entry, input, constant).
 __device__ __forceinline__ uint64_t leaf_value(const Dec& d, const DevProg& P, const DevState& S, uint32_t inst,
                                                uint64_t t, uint64_t key, const uint64_t* mir_cur) {
-    if (d.op == D_LDR) return load_reg(S, uint32_t(t & 1), d.c, d.b | (d.x << 16), inst);
+    if (d.op == D_LDR) return load_reg1(S, uint32_t(t & 1), d.c, d.b | (d.x << 16), inst);
     if (d.op == D_LDM) return mir_cur[d.b | (d.x << 16)];
     if (d.op == D_LDI) return stimulus(P, S, key, d.imm, inst, t, d.w);
     return (uint64_t)d.imm | ((uint64_t)d.a << 32) | ((uint64_t)d.b << 48);   // D_CONST
@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(1024) k_cycles_cl(DevProg P, DevState S, Launc
         const uint32_t lo = P.mir_off[blockIdx.x], hi = P.mir_off[blockIdx.x + 1];
         for (uint32_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
             const uint32_t r = P.mir_reg[i];
-            mirror[(uint64_t)par * A.mirror_words + (i - lo)] = load_reg(S, par, P.reg_cls[r], P.reg_idx[r], 0);
+            mirror[(uint64_t)par * A.mirror_words + (i - lo)] = load_reg1(S, par, P.reg_cls[r], P.reg_idx[r], 0);
         }
     }
     if (threadIdx.x == 0) {
@@ -653,8 +653,8 @@ __global__ void k_reset_slots(DevProg P, DevState S, uint32_t par, uint32_t lo, 
     for (uint64_t e = gtid; e < (uint64_t)P.n_reg * n; e += gth) {
         uint32_t r = uint32_t(e / n), inst = lo + uint32_t(e % n);
         uint32_t cls = P.reg_cls[r], idx = P.reg_idx[r];
-        if (cls == RC_W64) S.w64[par][(uint64_t)idx * S.I + inst] = reg_init[r];
-        else if (cls == RC_W32) S.w32[par][(uint64_t)idx * S.I + inst] = uint32_t(reg_init[r]);
+        if (cls == RC_W64) S.w64[par][reg_pos(S, S.n_w64, idx, inst)] = reg_init[r];
+        else if (cls == RC_W32) S.w32[par][reg_pos(S, S.n_w32, idx, inst)] = uint32_t(reg_init[r]);
     }
     for (uint64_t e = gtid; e < (uint64_t)P.n_reg * (w_hi - w_lo + 1); e += gth) {
         uint32_t r = uint32_t(e / (w_hi - w_lo + 1)), wi = w_lo + uint32_t(e % (w_hi - w_lo + 1));
@@ -662,7 +662,7 @@ __global__ void k_reset_slots(DevProg P, DevState S, uint32_t par, uint32_t lo, 
         uint32_t b0 = wi * S.pack, mask = 0;
         for (uint32_t b = 0; b < S.pack; b++)
             if (b0 + b >= lo && b0 + b < lo + n) mask |= 1u << b;
-        uint32_t* word = S.bits[par] + (uint64_t)P.reg_idx[r] * S.bit_stride + wi;
+        uint32_t* word = S.bits[par] + bit_pos(S, P.reg_idx[r], wi * S.pack);
         *word = (*word & ~mask) | ((reg_init[r] & 1) ? mask : 0u);
     }
     for (uint64_t e = gtid; e < mem_words * n; e += gth) {
@@ -679,6 +679,29 @@ __global__ void k_reset_slots(DevProg P, DevState S, uint32_t par, uint32_t lo, 
     for (uint64_t e = gtid; e < n; e += gth) const_cast<uint64_t*>(S.rom_dig)[lo + e] = rom_init_dig;
     for (uint64_t e = gtid; e < (uint64_t)P.n_in * n; e += gth)
         const_cast<uint8_t*>(S.hold_flag)[(e / n) * S.I + lo + e % n] = 0;
+}
+
+// Registers of buffer `par` between the kernels' tiles and the checkpoint's
+// order ([register][instance], 1-bit registers [register][group word]), which
+// uses buffer par ^ 1: its contents are dead between steps.
+__global__ void k_retile(DevState S, uint32_t par, uint32_t to_tiles) {
+    const uint64_t I = S.I, W = I / 32;
+    const uint64_t n64 = S.n_w64 * I, n32 = n64 + S.n_w32 * I, n1 = n32 + S.n_bit * W;
+    for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n1; e += (uint64_t)gridDim.x * blockDim.x) {
+        if (e < n64) {
+            const uint64_t q = reg_pos(S, S.n_w64, uint32_t(e / I), uint32_t(e % I));
+            if (to_tiles) S.w64[par][q] = S.w64[par ^ 1][e];
+            else S.w64[par ^ 1][e] = S.w64[par][q];
+        } else if (e < n32) {
+            const uint64_t j = e - n64, q = reg_pos(S, S.n_w32, uint32_t(j / I), uint32_t(j % I));
+            if (to_tiles) S.w32[par][q] = S.w32[par ^ 1][j];
+            else S.w32[par ^ 1][j] = S.w32[par][q];
+        } else {
+            const uint64_t j = e - n32, q = bit_pos(S, uint32_t(j / W), uint32_t(j % W) * 32u);
+            if (to_tiles) S.bits[par][q] = S.bits[par ^ 1][j];
+            else S.bits[par ^ 1][j] = S.bits[par][q];
+        }
+    }
 }
 
 // Full digest of buffer `par`: registers (part 0) and memory words (part 1),
@@ -843,6 +866,11 @@ cudaError_t launch_reset_slots(cudaStream_t st, const DevProg& P, const DevState
                                uint64_t mem_words, const uint64_t* mem_init_dig, uint64_t rom_init_dig) {
     k_reset_slots<<<256, 256, 0, st>>>(P, S, par, lo, n, reg_init, mem_image, mem_word_off, mem_words, mem_init_dig,
                                        rom_init_dig);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_retile(cudaStream_t st, const DevState& S, uint32_t par, bool to_tiles) {
+    k_retile<<<152 * 8, 256, 0, st>>>(S, par, to_tiles);
     return cudaGetLastError();
 }
 

@@ -30,6 +30,7 @@ cudaError_t launch_cycles_cl(bool digest, int grid, int threads, size_t smem, ui
                              const DevProg& P, const DevState& S, const LaunchArgs& A);
 cudaError_t launch_advance(cudaStream_t st, uint64_t* t0_dev, uint64_t n);
 cudaError_t launch_stim(cudaStream_t st, const DevProg& P, const DevState& S, uint64_t t, const uint64_t* t0_dev);
+cudaError_t launch_retile(cudaStream_t st, const DevState& S, uint32_t par, bool to_tiles);
 cudaError_t launch_set_u64(cudaStream_t st, uint64_t* p, uint64_t v);
 cudaError_t launch_state_digest(cudaStream_t st, const DevProg& P, const DevState& S, uint32_t par,
                                 const uint64_t* mem_word_off, uint64_t mem_words, uint64_t* out, uint32_t n_inst);
@@ -478,26 +479,34 @@ int ensure_loaded(sim_netlist* h, int mode, bool digest) {
     return SIM_OK;
 }
 
-// Launch plan for generated code: no shared memory, occupancy from registers.
-int plan_launch_gen(sim_batch* b) {
+// Warps per CTA and grid of generated code for b->n_tasks, on 1 / share of the
+// GPU.  Up to 1024 threads per CTA at 64 registers per thread.  Few tasks are
+// spread over the SMs in smaller CTAs (200k-op netlist, 304 tasks of 32
+// instances each: 24.3 us a cycle with 8 warps per CTA, 14.9 with 2; 64
+// instances: 18.2 with 8, 15.1 with 4); from 8 per SM on, 8 or more measured best.
+int plan_grid_gen(sim_batch* b, uint32_t share) {
     const int sms = sm_count();
-    const uint32_t n_proc = uint32_t(b->nl->part.procs.size());
-    b->n_tasks = b->mode == SIM_MODE_LANE_INST ? n_proc * (b->I / 32) : n_proc * b->I;
-    b->slot_words = 0;
-    b->prog_words = 0;
-    b->smem = 0;
-    // generated kernels: up to 1024 threads per CTA at 64 registers per thread
-    int warps = std::min(32, b->cfg.warps_per_cta ? int(b->cfg.warps_per_cta) : 8);
-    b->warps = warps;
-    b->threads = warps * 32;
+    const int spread = int(std::min<uint32_t>(8, std::max<uint32_t>(2, (b->n_tasks + sms - 1) / sms)));
+    b->warps = std::min(32, b->cfg.warps_per_cta ? int(b->cfg.warps_per_cta) : spread);
+    b->threads = b->warps * 32;
     int occ = 0;
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, b->gen_kernel[b->cfg.digest_capacity > 0],
                                                            b->threads, 0));
     if (occ < 1) return set_err(SIM_ERR_CAPACITY, "generated kernel does not fit on an SM");
     b->max_grid = occ * sms;
-    int need = int((b->n_tasks + warps - 1) / warps);
-    b->grid = std::max(1, std::min(need, b->max_grid));
+    const int need = int((b->n_tasks + b->warps - 1) / b->warps);
+    b->grid = std::max(1, std::min(need, std::max(1, b->max_grid / int(std::max(1u, share)))));
     return SIM_OK;
+}
+
+// Launch plan for generated code: no shared memory, occupancy from registers.
+int plan_launch_gen(sim_batch* b) {
+    const uint32_t n_proc = uint32_t(b->nl->part.procs.size());
+    b->n_tasks = b->mode == SIM_MODE_LANE_INST ? n_proc * (b->I / 32) : n_proc * b->I;
+    b->slot_words = 0;
+    b->prog_words = 0;
+    b->smem = 0;
+    return plan_grid_gen(b, 1);
 }
 
 // Keep the device copy of the state view (read by generated code) current.
@@ -700,10 +709,12 @@ int init_state(sim_batch* b) {
     DevState& S = b->S;
     S.I = b->I;
     S.pack = b->mode == SIM_MODE_LANE_INST ? 32 : 1;
-    S.bit_stride = uint32_t((I + S.pack - 1) / S.pack);
+    S.n_bit = L.count[RC_BIT];
+    S.n_w32 = L.count[RC_W32];
+    S.n_w64 = L.count[RC_W64];
     int rc;
     for (int k = 0; k < 2; k++) {
-        if ((rc = b->bits[k].alloc(size_t(L.count[RC_BIT]) * S.bit_stride * 4)) ||
+        if ((rc = b->bits[k].alloc(size_t(L.count[RC_BIT]) * (I / S.pack) * 4)) ||
             (rc = b->w32[k].alloc(size_t(L.count[RC_W32]) * I * 4)) || (rc = b->w64[k].alloc(size_t(L.count[RC_W64]) * I * 8)) ||
             (rc = b->rec[k].alloc(nl.wports.size() * I * 16)))
             return rc;
@@ -715,22 +726,35 @@ int init_state(sim_batch* b) {
     }
     // register planes of buffer 0 from init values (host-built, one plane at a time)
     {
-        std::vector<uint32_t> bitw(size_t(L.count[RC_BIT]) * S.bit_stride);
-        std::vector<uint32_t> w32(size_t(L.count[RC_W32]) * I);
-        std::vector<uint64_t> w64(size_t(L.count[RC_W64]) * I);
+        // one tile (lane = instance: 32 instances of every register), repeated for every group
+        const size_t row = S.pack == 32 ? 32 : size_t(I), tiles = size_t(I) / row, words = row / S.pack;
+        std::vector<uint32_t> bitw(size_t(L.count[RC_BIT]) * words);
+        std::vector<uint32_t> w32(size_t(L.count[RC_W32]) * row);
+        std::vector<uint64_t> w64(size_t(L.count[RC_W64]) * row);
         for (size_t r = 0; r < nl.reg_w.size(); r++) {
             uint64_t v = nl.reg_init[r];
             uint32_t ix = L.idx[r];
-            if (L.cls[r] == RC_W64) std::fill(w64.begin() + size_t(ix) * I, w64.begin() + size_t(ix + 1) * I, v);
-            else if (L.cls[r] == RC_W32) std::fill(w32.begin() + size_t(ix) * I, w32.begin() + size_t(ix + 1) * I, uint32_t(v));
+            if (L.cls[r] == RC_W64) std::fill_n(w64.begin() + size_t(ix) * row, row, v);
+            else if (L.cls[r] == RC_W32) std::fill_n(w32.begin() + size_t(ix) * row, row, uint32_t(v));
             else {
                 uint32_t word = (v & 1) ? (S.pack == 32 ? 0xffffffffu : 1u) : 0u;
-                std::fill(bitw.begin() + size_t(ix) * S.bit_stride, bitw.begin() + size_t(ix + 1) * S.bit_stride, word);
+                std::fill_n(bitw.begin() + size_t(ix) * words, words, word);
             }
         }
-        if (!bitw.empty()) CUDA_TRY(cudaMemcpyAsync(S.bits[0], bitw.data(), bitw.size() * 4, cudaMemcpyHostToDevice, st));
-        if (!w32.empty()) CUDA_TRY(cudaMemcpyAsync(S.w32[0], w32.data(), w32.size() * 4, cudaMemcpyHostToDevice, st));
-        if (!w64.empty()) CUDA_TRY(cudaMemcpyAsync(S.w64[0], w64.data(), w64.size() * 8, cudaMemcpyHostToDevice, st));
+        // the tile from the host, then copies of it on the device, doubling
+        auto spread = [&](void* dst, const void* tile, size_t bytes) -> int {
+            if (!bytes) return SIM_OK;
+            char* d = static_cast<char*>(dst);
+            CUDA_TRY(cudaMemcpyAsync(d, tile, bytes, cudaMemcpyHostToDevice, st));
+            for (size_t done = bytes, n; done < bytes * tiles; done += n) {
+                n = std::min(done, bytes * tiles - done);
+                CUDA_TRY(cudaMemcpyAsync(d + done, d, n, cudaMemcpyDeviceToDevice, st));
+            }
+            return SIM_OK;
+        };
+        if ((rc = spread(S.bits[0], bitw.data(), bitw.size() * 4)) || (rc = spread(S.w32[0], w32.data(), w32.size() * 4)) ||
+            (rc = spread(S.w64[0], w64.data(), w64.size() * 8)))
+            return rc;
         CUDA_TRY(cudaStreamSynchronize(st));
     }
     // memories
@@ -1048,15 +1072,23 @@ int check_inst(sim_batch* b, uint32_t inst) {
     return SIM_OK;
 }
 
+// Register planes (see reg_pos): register ix of an instance is at base + ix * row.
+uint64_t plane_row(const DevState& S) { return S.pack == 32 ? 32 : S.I; }
+uint64_t plane_base(const DevState& S, uint32_t n, uint32_t inst) {
+    return S.pack == 32 ? uint64_t(inst / 32) * n * 32 + inst % 32 : inst;
+}
+uint64_t bit_row(const DevState& S) { return S.pack == 32 ? 1 : S.I; }
+uint64_t bit_base(const DevState& S, uint32_t inst) { return S.pack == 32 ? uint64_t(inst / 32) * S.n_bit : inst; }
+
 // Address of register r of `inst` in buffer par (device pointer, element size, bit).
 void reg_addr(sim_batch* b, uint32_t par, uint32_t r, uint32_t inst, void** p, int* bytes, int* bit) {
     const RegLayout& L = b->nl->layout;
     uint64_t ix = L.idx[r];
     const DevState& S = b->S;
     *bit = -1;
-    if (L.cls[r] == RC_W64) { *p = S.w64[par] + ix * S.I + inst; *bytes = 8; }
-    else if (L.cls[r] == RC_W32) { *p = S.w32[par] + ix * S.I + inst; *bytes = 4; }
-    else { *p = S.bits[par] + ix * S.bit_stride + inst / S.pack; *bytes = 4; *bit = int(inst % S.pack); }
+    if (L.cls[r] == RC_W64) { *p = S.w64[par] + plane_base(S, S.n_w64, inst) + ix * plane_row(S); *bytes = 8; }
+    else if (L.cls[r] == RC_W32) { *p = S.w32[par] + plane_base(S, S.n_w32, inst) + ix * plane_row(S); *bytes = 4; }
+    else { *p = S.bits[par] + bit_base(S, inst) + ix * bit_row(S); *bytes = 4; *bit = int(inst % S.pack); }
 }
 
 }  // namespace
@@ -1331,13 +1363,13 @@ int sim_peek_regs(sim_batch* b, uint32_t inst, uint64_t* out) {
     std::vector<uint64_t> v64(L.count[RC_W64]);
     std::vector<uint32_t> v32(L.count[RC_W32]), v1(L.count[RC_BIT]);
     if (!v64.empty())
-        CUDA_TRY(cudaMemcpy2DAsync(v64.data(), 8, S.w64[par] + inst, size_t(S.I) * 8, 8, v64.size(),
+        CUDA_TRY(cudaMemcpy2DAsync(v64.data(), 8, S.w64[par] + plane_base(S, S.n_w64, inst), plane_row(S) * 8, 8, v64.size(),
                                    cudaMemcpyDeviceToHost, b->stream));
     if (!v32.empty())
-        CUDA_TRY(cudaMemcpy2DAsync(v32.data(), 4, S.w32[par] + inst, size_t(S.I) * 4, 4, v32.size(),
+        CUDA_TRY(cudaMemcpy2DAsync(v32.data(), 4, S.w32[par] + plane_base(S, S.n_w32, inst), plane_row(S) * 4, 4, v32.size(),
                                    cudaMemcpyDeviceToHost, b->stream));
     if (!v1.empty())
-        CUDA_TRY(cudaMemcpy2DAsync(v1.data(), 4, S.bits[par] + inst / S.pack, size_t(S.bit_stride) * 4, 4, v1.size(),
+        CUDA_TRY(cudaMemcpy2DAsync(v1.data(), 4, S.bits[par] + bit_base(S, inst), bit_row(S) * 4, 4, v1.size(),
                                    cudaMemcpyDeviceToHost, b->stream));
     CUDA_TRY(cudaStreamSynchronize(b->stream));
     for (size_t r = 0; r < L.cls.size(); r++) {
@@ -1417,8 +1449,13 @@ int sim_save(sim_batch* b, void** blob, size_t* len) {
     if (rc) return rc;
     const RegLayout& L = b->nl->layout;
     const DevState& S = b->S;
-    const uint32_t par = uint32_t(b->cycle & 1);
-    size_t nb = size_t(L.count[RC_BIT]) * S.bit_stride * 4, n32 = size_t(L.count[RC_W32]) * S.I * 4,
+    // registers in [register][instance] order whatever the kernels' layout
+    uint32_t par = uint32_t(b->cycle & 1);
+    if (S.pack == 32) {
+        CUDA_TRY(launch_retile(b->stream, S, par, false));
+        par ^= 1;
+    }
+    size_t nb = size_t(L.count[RC_BIT]) * (S.I / S.pack) * 4, n32 = size_t(L.count[RC_W32]) * S.I * 4,
            n64 = size_t(L.count[RC_W64]) * S.I * 8, nm = b->mem.n, nmd = b->mem_dig.n, nh = b->h_hold_val.size();
     size_t total = sizeof(BlobHeader) + nb + n32 + n64 + nm + nmd + nh * 9;
     char* p = static_cast<char*>(malloc(total));
@@ -1459,10 +1496,11 @@ int sim_restore(sim_batch* b, const void* blob, size_t len) {
     if (h.magic != kMagic || h.version != 1 || h.n_reg != b->nl->nl.reg_w.size() || h.I != S.I ||
         h.mode != uint64_t(b->mode) || h.n_mem_words != b->nl->mem_word_off.back())
         return set_err(SIM_ERR_BADARG, "checkpoint does not match this batch");
-    size_t nb = size_t(L.count[RC_BIT]) * S.bit_stride * 4, n32 = size_t(L.count[RC_W32]) * S.I * 4,
+    size_t nb = size_t(L.count[RC_BIT]) * (S.I / S.pack) * 4, n32 = size_t(L.count[RC_W32]) * S.I * 4,
            n64 = size_t(L.count[RC_W64]) * S.I * 8, nm = b->mem.n, nmd = b->mem_dig.n, nh = b->h_hold_val.size();
     if (len != sizeof h + nb + n32 + n64 + nm + nmd + nh * 9) return set_err(SIM_ERR_BADARG, "checkpoint size mismatch");
-    const uint32_t par = uint32_t(h.cycle & 1);
+    const bool tiled = S.pack == 32;
+    const uint32_t par = uint32_t(h.cycle & 1) ^ (tiled ? 1u : 0u);
     const char* q = static_cast<const char*>(blob) + sizeof h;
     auto h2d = [&](void* dst, size_t n) {
         if (n && b->h2d(dst, q, n) != SIM_OK) return false;
@@ -1471,6 +1509,7 @@ int sim_restore(sim_batch* b, const void* blob, size_t len) {
     };
     if (!h2d(S.bits[par], nb) || !h2d(S.w32[par], n32) || !h2d(S.w64[par], n64) || !h2d(S.mem, nm) || !h2d(S.mem_dig, nmd))
         return set_err(SIM_ERR_CUDA, "restore copy failed");
+    if (tiled) CUDA_TRY(launch_retile(b->stream, S, par ^ 1u, true));
     if (nh) {
         memcpy(b->h_hold_val.data(), q, nh * 8);
         q += nh * 8;
@@ -1647,6 +1686,7 @@ int pool_set_active(sim_batch* b, uint32_t n_groups, uint32_t share) {
     b->n_tasks = uint32_t(b->nl->part.procs.size()) * n_groups;
     // a persistent step holds only the CTAs its tasks need, and at most its
     // share of the GPU, leaving the other SMs to the pools of other netlists
+    if (b->generated) return plan_grid_gen(b, share);
     const int cap = std::max(1, b->max_grid / int(std::max(1u, share)));
     b->grid = std::max(1, std::min(int((b->n_tasks + b->warps - 1) / b->warps), cap));
     return SIM_OK;

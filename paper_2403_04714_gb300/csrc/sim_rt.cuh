@@ -80,11 +80,37 @@ static __device__ bool grid_barrier(uint32_t* bar, uint32_t& gen, uint64_t timeo
     return s_ok != 0;
 }
 
+// Position of register idx (of the n of its class) of an instance in its
+// plane.  With lane = instance a group's registers are contiguous, so that
+// generated code addresses each as one base plus a constant: with planes of
+// [register][all instances] every load and store first multiplied the register
+// by the batch's instance count, in 64 bits, and half of all instructions were
+// addresses (200k-op netlist x 4,096, 10 cycles: 759M -> 426M warp
+// instructions, 270 -> 186 us a cycle, 4.8 TB/s of DRAM traffic).  Bound by
+// that traffic (state, spills) and load latency; fetching a row ahead of its
+// use, into L1 or L2, measured no faster (184-196 us).
+__device__ __forceinline__ uint64_t reg_pos(const DevState& S, uint32_t n, uint32_t idx, uint32_t inst) {
+    if (S.pack == 32) return ((uint64_t)(inst >> 5) * n + idx) * 32u + (inst & 31u);
+    return (uint64_t)idx * S.I + inst;
+}
+
+// Word of 1-bit register idx that holds an instance.
+__device__ __forceinline__ uint64_t bit_pos(const DevState& S, uint32_t idx, uint32_t inst) {
+    return S.pack == 32 ? (uint64_t)(inst >> 5) * S.n_bit + idx : (uint64_t)idx * S.I + inst;
+}
+
 __device__ __forceinline__ uint64_t load_reg(const DevState& S, uint32_t par, uint32_t cls, uint32_t idx, uint32_t inst) {
+    if (cls == RC_W64) return S.w64[par][reg_pos(S, S.n_w64, idx, inst)];
+    if (cls == RC_W32) return S.w32[par][reg_pos(S, S.n_w32, idx, inst)];
+    uint32_t word = S.bits[par][bit_pos(S, idx, inst)];
+    return (word >> (inst % S.pack)) & 1u;
+}
+
+// The same for batches of one instance per warp (pack 1).
+__device__ __forceinline__ uint64_t load_reg1(const DevState& S, uint32_t par, uint32_t cls, uint32_t idx, uint32_t inst) {
     if (cls == RC_W64) return S.w64[par][(uint64_t)idx * S.I + inst];
     if (cls == RC_W32) return S.w32[par][(uint64_t)idx * S.I + inst];
-    uint32_t word = S.bits[par][(uint64_t)idx * S.bit_stride + inst / S.pack];
-    return (word >> (inst % S.pack)) & 1u;
+    return S.bits[par][(uint64_t)idx * S.I + inst] & 1u;
 }
 
 __device__ __forceinline__ uint64_t stimulus(const DevProg& P, const DevState& S, uint64_t key, uint32_t k, uint32_t inst,
@@ -185,9 +211,8 @@ static __device__ void final_commit(const DevProg& P, const DevState& S, uint64_
     }
 }
 
-// Input values of cycle t for every (input, instance), k-major so that the
-// lanes of a generated process function (consecutive instances) read
-// consecutive words: each input is hashed once per instance and cycle instead
+// Input values of cycle t for every (input, instance), laid out like the
+// registers: each input is hashed once per instance and cycle instead
 // of once in every process that reads it (about 80 processes per input on the
 // 200k-op netlist).  Grid-stride over the calling threads.
 __device__ __forceinline__ void fill_stim(const DevProg& P, const DevState& S, uint64_t t, uint64_t tid,
@@ -199,7 +224,7 @@ __device__ __forceinline__ void fill_stim(const DevProg& P, const DevState& S, u
     for (uint64_t e = tid; e < n; e += nth) {
         const uint32_t k = small ? uint32_t(e) / I : uint32_t(e / I);
         const uint32_t inst = small ? uint32_t(e) - k * I : uint32_t(e % I);
-        out[e] = stimulus(P, S, S.key[inst], k, inst, t, P.in_w[k]);
+        out[reg_pos(S, P.n_in, k, inst)] = stimulus(P, S, S.key[inst], k, inst, t, P.in_w[k]);
     }
 }
 
