@@ -86,6 +86,7 @@ struct DevProg {
     const uint8_t* reg_cls;
     const uint32_t* reg_idx;
     // cluster exchange (null unless the netlist was lowered for clusters)
+    const uint32_t* proc_order; // processes by descending cost (generated code, process-major order)
     const uint32_t* warp_proc;  // process of each warp of the grid, kNoProc if idle
     const uint32_t* mir_off;    // per CTA: first mirror entry (grid+1 offsets)
     const uint32_t* mir_reg;    // register held by each mirror entry

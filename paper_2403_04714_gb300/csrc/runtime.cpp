@@ -177,7 +177,8 @@ struct sim_batch {
     uint64_t seed = 0, cycle = 0;
     // program tables
     DBuf s_ins, s_off, s_len, c_words, c_off, c_size, b_ins, b_off, b_len, mport_off, mport_id, mem_lg, mem_w, mem_base,
-        in_w, reg_cls, reg_idx, mem_word_off, warp_proc, mir_off, mir_reg, warp_off, warp_slots;
+        in_w, reg_cls, reg_idx, mem_word_off, warp_proc, mir_off, mir_reg, warp_off, warp_slots,
+        proc_order;
     bool cluster = false;                   // cluster exchange kernel (k_cycles_cl)
     uint32_t mirror_off = 0;                // cluster CTA layout: mirror start (64-bit words)
     // state
@@ -670,7 +671,13 @@ int upload_program(sim_batch* b) {
         (rc = upload(b->mem_word_off, h->mem_word_off, st)) || (rc = upload(b->warp_proc, h->cplan.warp_proc, st)) ||
         (rc = upload(b->mir_off, h->cplan.mir_off, st)) || (rc = upload(b->mir_reg, h->cplan.mir_reg, st)))
         return rc;
+    std::vector<uint32_t> order(h->part.procs.size());
+    for (size_t p = 0; p < order.size(); p++) order[p] = uint32_t(p);
+    std::stable_sort(order.begin(), order.end(),
+                     [&](uint32_t x, uint32_t y) { return h->part.proc_cost[x] > h->part.proc_cost[y]; });
+    if ((rc = upload(b->proc_order, order, st))) return rc;
     DevProg& P = b->P;
+    P.proc_order = b->proc_order.as<uint32_t>();
     P.s_ins = b->s_ins.as<DIns>();
     P.s_off = b->s_off.as<uint32_t>();
     P.s_len = b->s_len.as<uint32_t>();
