@@ -64,6 +64,30 @@ constexpr uint32_t kChainMax = 2;
 constexpr uint32_t kStepCountMask = 0xffu;
 constexpr uint32_t kLeafStepMax = 128;
 
+// Operators of shared-memory programs as the interpreter runs them: every
+// operator is one formula over four operands A, M, X, D read from shared
+// memory, with constants of the formula in a table there, so that lanes with
+// different operators follow one short instruction path: with c = D != 0 ? X : M,
+//   h = and ? A & c : A ^ c,   f = or-c ? h | c : h,
+//   result = (A * M + f | A >> D | A << D) & mask,  or eq: f == 0,  lt: A < X,
+// where a shift that is off has bit 6 or 7 set in its amount (it gives 0) and
+// eq, lt have mask 0.  16 bytes: word 0 = lt | kOpMark | destination << 16, word 1 =
+// A | M << 16, word 2 = X | D << 16, word 3 = the bits below.  Operands and
+// destinations are byte offsets: below kOpSlot0 into the constant table, from
+// there on of a value slot; each warp adds its areas' places when it copies
+// its program (the mark tells these instructions from the others).
+constexpr uint32_t kOpMark = 1u << 7;         // never set in a DIns: its opcode is below 32
+constexpr uint32_t kOpSlot0 = 1024;
+constexpr uint32_t kOpLt = 1u << 0;            // word 0
+constexpr uint32_t kOpEq = 1u << 0;
+constexpr uint32_t kOpChainA = 1u << 2, kOpChainX = 1u << 3, kOpChainD = 1u << 4;   // operand = the lane's first result
+constexpr uint32_t kOpInv = 1u << 5;          // second rows: c = D == 0 ? X : M
+constexpr uint32_t kOpNoShr = 1u << 6, kOpNoShl = 1u << 7;
+constexpr uint32_t kOpAnd = 1u << 15, kOpOrC = 1u << 23;   // sign bits of their bytes
+constexpr uint32_t kOpMaskShift = 25;         // 64 - width (64: mask 0)
+// Constant table (64-bit words): 0, ~0, the powers of two, then 3, 5, 6, 7, 9, ... 63.
+constexpr uint32_t kTabZero = 0, kTabOnes = 1, kTabPow2 = 2, kTabInts = 66, kTabWords = 124;
+
 
 
 // Program tables of one lowered netlist (device pointers).
@@ -71,9 +95,10 @@ struct DevProg {
     const DIns* s_ins;          // LANE_OP bundles (32 instructions per row)
     const uint32_t* s_off;
     const uint32_t* s_len;
-    const uint32_t* c_words;    // LANE_OP compact programs (step table + instructions)
+    const uint32_t* e_words;    // LANE_OP shared-memory programs (step table + instructions)
     const uint32_t* c_off;      // per process: first word
     const uint32_t* c_size;     // per process: words (multiple of 4)
+    const uint32_t* e_tab;      // per process: 16-byte units of the step table
     const DIns* b_ins;          // LANE_INST linear streams
     const uint32_t* b_off;
     const uint32_t* b_len;
@@ -91,7 +116,8 @@ struct DevProg {
     const uint32_t* mir_off;    // per CTA: first mirror entry (grid+1 offsets)
     const uint32_t* mir_reg;    // register held by each mirror entry
     const uint32_t* warp_off;   // per warp: start of its slots in its CTA's shared memory (64-bit words)
-    const uint32_t* warp_slots; // per warp: its slot words, the last one spare (program follows)
+    const uint32_t* warp_slots; // per warp: its slot words, the last one spare
+    const uint32_t* warp_prog;  // per warp: start of its program (64-bit words)
     uint32_t n_proc, n_in, n_reg, n_mem, n_wport;
 };
 
@@ -137,6 +163,7 @@ struct LaunchArgs {
     uint32_t warps_per_cta;
     uint32_t slot_words;        // per-warp slot area in 64-bit words (even)
     uint32_t prog_words;        // per-warp resident program area in 32-bit words (0 = read from global)
+    uint32_t replicas;          // LANE_OP: warps per process, each with its share of the instances
     uint32_t n_tasks;           // processes x instance groups
     uint32_t group;             // instances per task (1 LANE_OP, 32 LANE_INST)
     uint32_t proc_major;        // process-major task order (in waves), else group-major

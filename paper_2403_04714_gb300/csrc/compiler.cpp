@@ -1425,6 +1425,23 @@ struct SlotAlloc {
 
 namespace {
 
+// Operators that never run in operator or chain steps: memory reads, and
+// shifts by an amount of more than 32 bits (the step interpreter's shifts read
+// 32 bits of it).
+bool generic_op(const Netlist& nl, int32_t id) {
+    const Node& d = nl.nodes[id];
+    return d.op == OP_MEMRD || ((d.op == OP_SHL || d.op == OP_SHR) && nl.nodes[d.b].w > 32);
+}
+
+// The second operator of a pair takes its first result at most once as a
+// factor, and as only one of a mux's two values (encode_op).
+bool pair_fits(const Netlist& nl, int32_t id, int32_t prev) {
+    const Node& d = nl.nodes[id];
+    if (d.op == OP_MUL) return !(d.a == prev && d.b == prev);
+    if (d.op == OP_MUX) return !(d.b == prev && d.c == prev);
+    return true;
+}
+
 // One step of a shared-memory program.
 struct CStep {
     uint32_t flags = 0;
@@ -1491,7 +1508,7 @@ int chained_program(const Netlist& nl, const std::vector<Item>& items, const std
     std::vector<uint8_t> has_memrd, has_chain;
     std::vector<int32_t> deps;
     for (size_t k = 0; k < no; k++) {
-        const bool memrd = nl.nodes[items[opers[k]].id].op == OP_MEMRD;
+        const bool memrd = generic_op(nl, items[opers[k]].id);
         deps.clear();
         operands(items[opers[k]], [&](int32_t n) {
             const int32_t q = op_of_local[local[n]];
@@ -1502,7 +1519,8 @@ int chained_program(const Netlist& nl, const std::vector<Item>& items, const std
         bool placed = false;
         if (!memrd && s > 0 && !has_memrd[s - 1])
             for (int32_t d : deps) {
-                if (ostep[d] != s - 1 || nl.nodes[items[opers[d]].id].op == OP_MEMRD) continue;
+                if (ostep[d] != s - 1 || generic_op(nl, items[opers[d]].id)) continue;
+                if (!pair_fits(nl, items[opers[k]].id, items[opers[d]].id)) continue;
                 auto& L = lanes[s - 1][olane[d]];
                 if (L.back() != d || L.size() >= K) continue;
                 bool ok = true;
@@ -1743,6 +1761,7 @@ int lower(const Netlist& nl, const Partition& part, Lowered& out, std::string& e
                     d.op = uint8_t(D_ADD + (n.op - OP_ADD));
                     d.a = S(n.a);
                     d.b = S(n.b);
+                    if (n.op == OP_SHL || n.op == OP_SHR) d.x = generic_op(nl, it.id);   // a generic step's operator
                 }
             } else if (it.kind == 1) {
                 int32_t r = it.id;
@@ -1809,14 +1828,15 @@ int lower(const Netlist& nl, const Partition& part, Lowered& out, std::string& e
             std::vector<CStep> steps;
             for (uint32_t b = 0; b < nb; b++) {
                 const DIns* row = &out.s_ins[(size_t(out.s_off[p]) + b) * 32];
-                bool operators_only = true, leaves_only = count[b] > 0, stores_only = count[b] > 0;
+                bool wide_shift = false, operators_only = true, leaves_only = count[b] > 0, stores_only = count[b] > 0;
                 for (uint32_t l = 0; l < count[b]; l++) {
                     operators_only &= row[l].op >= D_ADD && row[l].op <= D_CONCAT;
+                    wide_shift |= (row[l].op == D_SHL || row[l].op == D_SHR) && row[l].x;
                     leaves_only &= row[l].op == D_LDR || row[l].op == D_LDI || row[l].op == D_CONST;
                     stores_only &= row[l].op == D_STR;
                 }
                 const uint32_t wide = leaves_only ? kStepLeaf : stores_only ? kStepStore : 0u;
-                const uint32_t flags = (operators_only ? 0u : kStepGeneric) | wide;
+                const uint32_t flags = (operators_only && !wide_shift ? 0u : kStepGeneric) | wide;
                 if (wide && !steps.empty() && (steps.back().flags & wide) &&
                     steps.back().ins.size() + count[b] <= kLeafStepMax) {
                     steps.back().ins.insert(steps.back().ins.end(), row, row + count[b]);
@@ -1912,6 +1932,95 @@ int lower(const Netlist& nl, const Partition& part, Lowered& out, std::string& e
     return SIM_OK;
 }
 
+
+// ---------------------------------------------------------------------------
+// Device form of the compact programs
+// ---------------------------------------------------------------------------
+namespace {
+
+uint32_t tab(uint32_t i) { return i * 8; }
+uint32_t tab_pow2(uint32_t k) { return tab(kTabPow2 + k); }
+// the constant v of 0..64
+uint32_t tab_int(uint32_t v) {
+    if (v == 0) return tab(kTabZero);
+    uint32_t lg = 0;
+    while ((2u << lg) <= v) lg++;
+    if (v == 1u << lg) return tab_pow2(lg);
+    return tab(kTabInts + v - 2 - lg);      // lg + 1 powers of two lie below v
+}
+
+void encode_op(const DIns& d, bool second, uint32_t out[4]) {
+    const auto S = [](uint16_t s) { return kOpSlot0 + uint32_t(s) * 8; };
+    const uint32_t zero = tab(kTabZero);
+    uint32_t A = zero, M = zero, X = zero, D = tab_int(64), bits = kOpNoShr | kOpNoShl;
+    uint32_t width = 64u - d.w;
+    const bool pa = second && (d.imm & 1u), pb = second && (d.imm & 2u), pc = second && (d.imm & 4u);
+    const auto chain = [&](bool on, uint32_t bit) { bits |= on ? bit : 0; };
+    switch (d.op) {
+    case D_ADD: case D_CONCAT:
+        A = S(d.a), X = S(d.b), M = tab_pow2(d.op == D_CONCAT ? d.x : 0);
+        bits |= kOpAnd | kOpOrC;
+        chain(pa, kOpChainA), chain(pb, kOpChainX);
+        break;
+    case D_SUB:                                   // b * ~0 + a
+        A = S(d.b), X = S(d.a), M = tab(kTabOnes);
+        bits |= kOpAnd | kOpOrC;
+        chain(pb, kOpChainA), chain(pa, kOpChainX);
+        break;
+    case D_MUL:
+        A = S(pb ? d.b : d.a), M = S(pb ? d.a : d.b);
+        bits |= kOpAnd;
+        chain(pa || pb, kOpChainA);
+        break;
+    case D_AND: case D_OR: case D_XOR: case D_EQ: case D_LT:
+        A = S(d.a), X = S(d.b);
+        bits |= d.op == D_AND ? kOpAnd : d.op == D_OR ? kOpOrC : d.op == D_EQ ? kOpEq : 0;
+        if (d.op == D_EQ || d.op == D_LT) width = 64;
+        chain(pa, kOpChainA), chain(pb, kOpChainX);
+        break;
+    case D_SHL: case D_SHR: case D_SLICE:
+        A = S(d.a), D = d.op == D_SLICE ? tab_int(d.x) : S(d.b);
+        bits |= kOpAnd;
+        bits &= ~(d.op == D_SHL ? kOpNoShl : kOpNoShr);
+        chain(pa, kOpChainA), chain(pb, kOpChainD);
+        break;
+    case D_MUX:                                   // 0 * M + (0 ^ c)
+        D = S(d.a), X = S(pc ? d.c : d.b), M = S(pc ? d.b : d.c);
+        chain(pa, kOpChainD), chain(pb || pc, kOpChainX), chain(pc, kOpInv);
+        break;
+    default:                                      // D_NOP: nothing (its result goes to the spare slot)
+        width = 64;
+        break;
+    }
+    out[0] = (d.op == D_LT ? kOpLt : 0u) | kOpMark | (d.op == D_NOP ? 0u : S(d.dst)) << 16;
+    out[1] = A | M << 16;
+    out[2] = X | D << 16;
+    out[3] = bits | width << kOpMaskShift;
+}
+
+}  // namespace
+
+void encode_programs(Lowered& low) {
+    low.e_words = low.c_words;
+    low.e_tab.assign(low.c_off.size(), 0);
+    for (size_t p = 0; p < low.c_off.size(); p++) {
+        const uint32_t* w = low.c_words.data() + low.c_off[p];
+        const uint32_t nb = w[0], tw = (nb + 4) & ~3u;
+        const DIns* ins = reinterpret_cast<const DIns*>(w + tw);
+        uint32_t* out = low.e_words.data() + low.c_off[p] + tw;
+        low.e_tab[p] = tw / 4;
+        for (uint32_t b = 0; b < nb; b++) {
+            const uint32_t e = w[1 + b], first = e & 0xffff, cnt = (e >> 16) & kStepCountMask;
+            const bool pair = e & kStepChain;
+            if (!pair && (e & kStepGeneric)) continue;
+            // a lane's two operators side by side; step words hold the last lane
+            const uint32_t n = pair ? cnt / 2 : cnt;
+            for (uint32_t i = 0; i < cnt; i++)
+                encode_op(ins[first + i], i >= n, out + size_t(first + (pair ? i % n * 2 + i / n : i)) * 4);
+            low.e_words[low.c_off[p] + 1 + b] = (e & ~(kStepCountMask << 16)) | (n - 1) << 16;
+        }
+    }
+}
 
 // ---------------------------------------------------------------------------
 // Cluster placement and exchange lowering

@@ -104,6 +104,9 @@ struct Lowered {
     std::vector<uint32_t> c_words;    // packed programs, 32-bit words
     std::vector<uint32_t> c_off;      // per process: first word (multiple of 4)
     std::vector<uint32_t> c_size;     // per process: words (multiple of 4)
+    // the compact programs as the device runs them (encode_programs), laid out
+    // like c_words; e_tab: 16-byte units before the instructions
+    std::vector<uint32_t> e_words, e_tab;
     // LANE_INST: linear instruction list
     std::vector<DIns> b_ins;
     std::vector<uint32_t> b_off, b_len, b_slots;
@@ -114,6 +117,12 @@ struct Lowered {
 // chain = 2: the compact programs run dependent operator pairs in one step
 // (one lane, the first result kept in a register); otherwise one level per step.
 int lower(const Netlist& nl, const Partition& part, Lowered& out, std::string& err, uint32_t chain = 0);
+
+// The device form of the compact programs: the operators of operator and chain
+// steps as instances of one formula (kOpMark), a chain step's pairs side by
+// side, and those steps' words with the number of their last lane in place of
+// the instruction count; everything else as it is.
+void encode_programs(Lowered& low);
 
 // Cluster exchange.  Processes are placed on a grid of thread-block
 // clusters (C CTAs of W warps, one process per warp) so that producers and

@@ -233,13 +233,12 @@ static __device__ bool cluster_barrier(uint64_t* bars, uint32_t c, uint32_t C, u
 // ---------------------------------------------------------------------------
 // LANE_OP: one warp, one process, one instance; lanes run a 32-wide step.
 // ---------------------------------------------------------------------------
-// All 13 operators without branches: every candidate result is formed and the
-// opcode selects one, so lanes running different operators in one schedule
-// step follow a single instruction path (no serialised divergent paths).  One
-// left and one right shift serve the four shift-like operators (the amount is
-// b for shl/shr and the static x for slice/concat), and add/sub share one
-// adder (b complemented with a carry in for sub); a select tree on the bits of
-// op - D_ADD (operators in enum order) picks the result in four levels.
+// All 13 operators without branches, for the rare operators outside operator
+// and pair steps (a step with a memory read, a shift by a wide amount) and for
+// programs in global memory.  One left and one right shift serve the four
+// shift-like operators, add/sub share one adder (b complemented with a carry
+// in for sub); a select tree on the bits of op - D_ADD (operators in enum
+// order) picks the result in four levels.
 __device__ __forceinline__ uint64_t alu_select(uint32_t op, uint64_t a, uint64_t b, uint64_t c, uint32_t x) {
     const uint32_t k = op - D_ADD;
     const bool k0 = k & 1u, k1 = k & 2u, k2 = k & 4u, k3 = k & 8u;
@@ -364,82 +363,171 @@ __device__ void task_lane_op(const DevProg& P, const DevState& S, uint32_t p, ui
     finish_lane_op<DIGEST>(S, p, inst, t, col, lane, dacc);
 }
 
-// Result of one operator instruction, reduced to its width.
-__device__ __forceinline__ uint64_t eval_op(const Dec& d, uint64_t a, uint64_t b, uint64_t c) {
-    return alu_select(d.op, a, b, c, d.x) & wmask(d.w);
+// One operator of a shared-memory program (abi_device.h has the formula).
+// Bound by the issue of its dependent instructions, one warp per scheduler
+// most of the time and about five lanes with an operator each; so it forms no
+// candidate that a constant operand can switch off instead, and the next
+// step's operators are loaded while this one's are evaluated.  200k-op netlist,
+// one instance, against a select tree over every operator's result: 12.3 ->
+// 9.0 us a cycle on the grid barrier (63 steps; 11.0 without the early load),
+// 10.5 -> 9.1 with operator pairs in 2-CTA clusters (38 steps), 499k-op mesh
+// 15.9 -> 10.5, 2k-op netlist in one cluster 3.8 -> 3.2.  Measured slower:
+// A == X and A < c from the selected operand (2 %), the result of a compare
+// selected in 64 bits (2-4 %), fields read as 16-bit words (3-5 %), the fields
+// taken apart before the warp barrier (no change), the mask as two shifts (5 %).
+// 64-bit shifts by 64 or more give 0, as PTX defines them.
+__device__ __forceinline__ uint64_t shr64(uint64_t v, uint32_t n) {
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
 }
 
-// Program resident in shared memory: `prog` holds the step count, the step
-// table (first instruction | count << 16 | flags) and, 16-byte aligned, the
-// instructions.  Operator-only steps run on all 32 lanes without a branch:
-// lanes past the step's count repeat its first instruction and write the
-// spare slot `dummy` (the last word of the warp's slot region), which no
-// instruction reads.
+__device__ __forceinline__ uint64_t shl64(uint64_t v, uint32_t n) {
+    uint64_t r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+}
+
+// All bits of the result: the sign bit of byte BYTE of v.
+template <int BYTE>
+__device__ __forceinline__ uint64_t byte_sign(uint32_t v) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(v), "n"(0x8888 + 0x1111 * BYTE));
+    return (uint64_t)r << 32 | r;
+}
+
+struct OpFields {
+    uint32_t a, m, x, d, dst, w0, bits;
+};
+
+__device__ __forceinline__ OpFields op_fields(uint4 o) {
+    return {o.y & 0xffffu, o.y >> 16, o.z & 0xffffu, o.z >> 16, o.x >> 16, o.x, o.w};
+}
+
+__device__ __forceinline__ uint64_t eval_op(uint32_t w0, uint32_t bits, uint64_t a, uint64_t m, uint64_t x, uint64_t d, bool inv) {
+    const uint64_t k_and = byte_sign<1>(bits), k_orx = byte_sign<2>(bits);
+    const bool P = (d != 0) != inv;
+    const uint64_t c = P ? x : m;
+    const uint64_t h = (a & c & k_and) | ((a ^ c) & ~k_and);
+    const uint64_t f = h | (c & k_orx);
+    const uint64_t t = a * m + f;
+    const uint32_t n = uint32_t(d);
+    const uint64_t s = shr64(a, n | (bits & kOpNoShr)) | shl64(a, n | (bits & kOpNoShl));
+    const uint32_t cmp = ((f == 0 ? bits : 0u) | (a < x ? w0 : 0u)) & 1u;
+    const uint64_t r = (t | s) & shr64(~0ull, bits >> kOpMaskShift);
+    return (r & 0xffffffff00000000ull) | (uint32_t(r) | cmp);
+}
+
+// Copies a process's program into the warp's area, adding the places of the
+// warp's slots (byte offset `slots` of dynamic shared memory) to the operators'
+// fields; a destination of 0 is the spare slot.
+__device__ __forceinline__ void copy_program(const DevProg& P, uint32_t p, uint32_t* prog, uint32_t slots, uint32_t spare,
+                                             uint32_t lane) {
+    const uint4* src = reinterpret_cast<const uint4*>(P.e_words + P.c_off[p]);
+    uint4* dst = reinterpret_cast<uint4*>(prog);
+    const uint32_t n = P.c_size[p] / 4, ni = P.e_tab[p];
+    const auto place = [&](uint32_t f) { return f < kOpSlot0 ? f : f - kOpSlot0 + slots; };
+    for (uint32_t k = lane; k < n; k += 32) {
+        uint4 v = __ldg(src + k);
+        if (k >= ni && (v.x & kOpMark)) {
+            const uint32_t to = v.x >> 16;
+            v.x = (v.x & 0xffff) | (to ? place(to) : spare) << 16;
+            v.y = place(v.y & 0xffff) | place(v.y >> 16) << 16;
+            v.z = place(v.z & 0xffff) | place(v.z >> 16) << 16;
+        }
+        dst[k] = v;
+    }
+}
+
+__device__ __forceinline__ void fill_const_table(uint64_t* tab) {
+    for (uint32_t i = threadIdx.x; i < kTabWords; i += blockDim.x) {
+        uint64_t v = i == kTabOnes ? ~0ull : 0ull;
+        if (i >= kTabPow2 && i < kTabInts) v = 1ull << (i - kTabPow2);
+        if (i >= kTabInts) {                     // entry of v: kTabInts + v - 2 - floor(log2 v)
+            v = i - kTabInts + 3;
+            for (uint32_t lg = 1; lg < 6; lg++) v += v >= (2u << lg) ? 1 : 0;
+        }
+        tab[i] = v;
+    }
+}
+
+// Program resident in shared memory (copy_program); `sm` is the start of
+// dynamic shared memory, `sl` the warp's slots, `dummy` its spare slot, which
+// no instruction reads (idle lanes of leaf steps write it).  Operator and pair
+// steps run on all 32 lanes without a branch: lanes past the step's last
+// repeat that lane's operators and store the same values.
 // PAIRS: the program was lowered with operator pairs, whose steps are tested
 // first (a program without them never pays that test).
 template <bool DIGEST, bool PAIRS>
 __device__ void task_lane_op_res(const DevProg& P, const DevState& S, uint32_t p, uint32_t inst, uint64_t t,
-                                 bool pending, uint64_t* __restrict__ sl, const uint32_t* __restrict__ prog,
-                                 uint32_t lane, uint32_t dummy, const uint64_t* mir_cur = nullptr,
-                                 uint32_t mir_nxt = 0) {
+                                 bool pending, char* sm, uint64_t* sl, const uint32_t* __restrict__ prog,
+                                 uint32_t lane, uint32_t dummy,
+                                 const uint64_t* mir_cur = nullptr, uint32_t mir_nxt = 0) {
     const uint64_t key = S.key[inst];
     const int32_t col = DIGEST ? S.track[inst] : -1;
     uint64_t dacc = 0;
     const uint32_t nb = prog[0];
+    // (the word after the last step word is padding or a leaf's first word: no chain bit)
     const uint32_t* table = prog + 1;
     const uint4* ins = reinterpret_cast<const uint4*>(prog + ((nb + 4) & ~3u));
-    uint32_t e = nb ? table[0] : 0;
+    const auto ld = [&](uint32_t off) { return *reinterpret_cast<const uint64_t*>(sm + off); };
+    const auto st = [&](uint32_t off, uint64_t v) { *reinterpret_cast<uint64_t*>(sm + off) = v; };
+    uint32_t e = table[0];
     for (uint32_t b = 0; b < nb;) {
         if (PAIRS) {
             // a run of pair steps (most of a pair program) in a loop of its own:
             // no step-kind dispatch on this path
-            while (e & kStepChain) {
-                // two rows: each lane's first operator, then its second one (no
-                // warp barrier between them); imm bits 0/1/2 take operands
-                // a/b/c of the second from the first result.  The second row's
-                // slot operands hold values of earlier steps (a slot written in
-                // this step is never read here except through the flags), so
-                // they are loaded together with the first row's, before its
-                // store.
-                const uint32_t e_next = b + 1 < nb ? table[b + 1] : 0;
-                const uint32_t first = e & 0xffff, n = ((e >> 16) & kStepCountMask) >> 1;
-                const bool on = lane < n;
-                const uint32_t i1 = on ? first + lane : first;
-                const Dec d1 = decode(ins[i1]);
-                const Dec d2 = decode(ins[i1 + n]);
-                const uint64_t a1 = sl[d1.a], b1 = sl[d1.b], c1 = sl[d1.c];
-                const uint64_t a2s = sl[d2.a], b2s = sl[d2.b], c2s = sl[d2.c];
-                const uint64_t r1 = eval_op(d1, a1, b1, c1);
-                const uint64_t r2 = eval_op(d2, (d2.imm & 1u) ? r1 : a2s, (d2.imm & 2u) ? r1 : b2s,
-                                            (d2.imm & 4u) ? r1 : c2s);
-                sl[on ? d1.dst : dummy] = r1;
-                sl[on && d2.op != D_NOP ? d2.dst : dummy] = r2;
-                __syncwarp();
-                e = e_next;
-                b++;
+            if (e & kStepChain) {
+                const uint4* o = ins + (e & 0xffff) + 2 * min(lane, (e >> 16) & 31u);
+                uint4 o1 = o[0], o2 = o[1];
+                do {
+                    // two rows: each lane's first operator, then its second one
+                    // (no warp barrier between them).  The second row's slot
+                    // operands hold values of earlier steps (a slot written in
+                    // this step is never read here except through the chain
+                    // bits), so they are loaded together with the first row's,
+                    // before its store; so are the next step's operators.
+                    e = table[++b];
+                    const OpFields f1 = op_fields(o1), f2 = op_fields(o2);
+                    const uint64_t a1 = ld(f1.a), m1 = ld(f1.m), x1 = ld(f1.x), d1 = ld(f1.d);
+                    const uint64_t a2 = ld(f2.a), m2 = ld(f2.m), x2 = ld(f2.x), d2 = ld(f2.d);
+                    o = (e & kStepChain) ? ins + (e & 0xffff) + 2 * min(lane, (e >> 16) & 31u) : o;
+                    const uint4 n1 = o[0], n2 = o[1];
+                    const uint64_t r1 = eval_op(f1.w0, f1.bits, a1, m1, x1, d1, false);
+                    st(f1.dst, r1);
+                    const uint64_t r2 = eval_op(f2.w0, f2.bits, (f2.bits & kOpChainA) ? r1 : a2, m2,
+                                                (f2.bits & kOpChainX) ? r1 : x2, (f2.bits & kOpChainD) ? r1 : d2,
+                                                f2.bits & kOpInv);
+                    st(f2.dst, r2);
+                    __syncwarp();
+                    o1 = n1;
+                    o2 = n2;
+                } while (e & kStepChain);
             }
             if (b >= nb) break;
         } else {
-            // a run of operator steps in a loop of its own likewise
-            while (!(e & kStepGeneric) && b < nb) {
-                const uint32_t e_next = b + 1 < nb ? table[b + 1] : 0;
-                const uint32_t first = e & 0xffff, cnt = (e >> 16) & kStepCountMask;
-                const bool on = lane < cnt;
-                const Dec d = decode(ins[on ? first + lane : first]);
-                sl[on ? d.dst : dummy] = eval_op(d, sl[d.a], sl[d.b], sl[d.c]);
-                __syncwarp();
-                e = e_next;
-                b++;
+            // a run of operator steps in a loop of its own likewise (the last
+            // step of a program holds stores)
+            if (!(e & kStepGeneric)) {
+                uint32_t i = (e & 0xffff) + min(lane, (e >> 16) & 31u);
+                uint4 o = ins[i];
+                do {
+                    e = table[++b];
+                    const OpFields f = op_fields(o);
+                    const uint64_t a = ld(f.a), m = ld(f.m), x = ld(f.x), d = ld(f.d);
+                    i = !(e & kStepGeneric) ? (e & 0xffff) + min(lane, (e >> 16) & 31u) : i;
+                    const uint4 n = ins[i];
+                    st(f.dst, eval_op(f.w0, f.bits, a, m, x, d, false));
+                    __syncwarp();
+                    o = n;
+                } while (!(e & kStepGeneric));
             }
-            if (b >= nb) break;
         }
-        const uint32_t e_next = b + 1 < nb ? table[b + 1] : 0;
+        const uint32_t e_next = table[b + 1];
         const uint32_t first = e & 0xffff, cnt = (e >> 16) & kStepCountMask;
-        if (!(e & kStepGeneric)) {
-            // operator step: all 32 lanes, no branch (idle lanes write the spare slot)
-            const bool on = lane < cnt;
-            const Dec d = decode(ins[on ? first + lane : first]);
-            sl[on ? d.dst : dummy] = eval_op(d, sl[d.a], sl[d.b], sl[d.c]);
+        if (PAIRS && !(e & kStepGeneric)) {
+            const OpFields f = op_fields(ins[first + min(lane, cnt)]);      // operator step
+            st(f.dst, eval_op(f.w0, f.bits, ld(f.a), ld(f.m), ld(f.x), ld(f.d), false));
         } else if (!PAIRS && (e & kStepStore)) {
             // programs without pairs: up to four register or mirror stores per
             // lane, every slot value loaded before the first store
@@ -495,19 +583,24 @@ __global__ void __launch_bounds__(1024) k_cycles(DevProg P, DevState S, LaunchAr
     const uint32_t lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const uint32_t warp = blockIdx.x * A.warps_per_cta + wib;
     const uint32_t tw = gridDim.x * A.warps_per_cta;
-    uint64_t* sl = smem + (uint64_t)wib * (A.slot_words + A.prog_words / 2);
-    uint32_t* prog = reinterpret_cast<uint32_t*>(sl + A.slot_words);
     const bool resident = MODE == SIM_MODE_LANE_OP && A.prog_words > 0;
+    // resident programs: the constant table, every warp's slots, then the programs
+    const uint32_t slot0 = (resident ? kTabWords : 0) + wib * A.slot_words;
+    uint64_t* sl = smem + slot0;
+    uint32_t* prog = reinterpret_cast<uint32_t*>(smem + kTabWords + A.warps_per_cta * A.slot_words) + wib * A.prog_words;
+    // warps beyond one per process repeat the processes for other instances
+    const uint32_t p_first = A.replicas > 1 ? warp % P.n_proc : warp, g_first = A.replicas > 1 ? warp / P.n_proc : 0;
+    const uint32_t p_step = A.replicas > 1 ? P.n_proc : tw;
+    const uint32_t spare = (slot0 + A.slot_words - 1) * 8;
     if (resident) {
-        // copy the compact programs of the processes this warp owns (p = warp + k*tw)
+        fill_const_table(smem);
+        // copy the programs of the processes this warp owns
         uint32_t off = 0;
-        for (uint32_t p = warp; p < P.n_proc; p += tw) {
-            const uint4* src = reinterpret_cast<const uint4*>(P.c_words + P.c_off[p]);
-            uint4* dst = reinterpret_cast<uint4*>(prog + off);
-            for (uint32_t k = lane; k < P.c_size[p] / 4; k += 32) dst[k] = __ldg(src + k);
+        for (uint32_t p = p_first; p < P.n_proc && g_first < A.replicas; p += p_step) {
+            copy_program(P, p, prog + off, slot0 * 8, spare, lane);
             off += P.c_size[p];
         }
-        __syncwarp();
+        __syncthreads();
     }
     const uint64_t t_base = A.t0_dev ? *A.t0_dev + A.t0 : A.t0;
     uint32_t gen = 0;
@@ -518,9 +611,10 @@ __global__ void __launch_bounds__(1024) k_cycles(DevProg P, DevState S, LaunchAr
         if (rec && threadIdx.x == 0) rec[0] = globaltimer_ns();
         if (resident) {
             uint32_t off = 0;
-            for (uint32_t p = warp; p < P.n_proc; p += tw) {
-                for (uint32_t g = 0; g < S.I; g++)
-                    task_lane_op_res<DIGEST, PAIRS>(P, S, p, g, t, pending, sl, prog + off, lane, A.slot_words - 1);
+            for (uint32_t p = p_first; p < P.n_proc && g_first < A.replicas; p += p_step) {
+                for (uint32_t g = g_first; g < S.I; g += A.replicas)
+                    task_lane_op_res<DIGEST, PAIRS>(P, S, p, g, t, pending, reinterpret_cast<char*>(smem), sl, prog + off,
+                                                    lane, A.slot_words - 1);
                 off += P.c_size[p];
             }
         } else {
@@ -564,16 +658,17 @@ __global__ void __launch_bounds__(1024) k_cycles_cl(DevProg P, DevState S, Launc
     }
     const uint32_t lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const uint32_t warp = blockIdx.x * A.warps_per_cta + wib;
-    // warps' areas packed by their own process's needs (slots, then program)
-    const uint32_t slot_words = P.warp_slots[warp];
-    uint64_t* sl = smem + P.warp_off[warp];
-    uint32_t* prog = reinterpret_cast<uint32_t*>(sl + slot_words);
+    // the constant table, then the warps' slots and their programs, packed by
+    // their own process's needs
+    const uint32_t slot_words = P.warp_slots[warp], slot0 = P.warp_off[warp];
+    const uint32_t spare = (slot0 + slot_words - 1) * 8;
+    uint64_t* sl = smem + slot0;
+    uint32_t* prog = reinterpret_cast<uint32_t*>(smem + P.warp_prog[warp]);
+    fill_const_table(smem);
     uint64_t* mirror = smem + A.mirror_off;
     const uint32_t p = P.warp_proc[warp];
     if (p != kNoProc) {
-        const uint4* src = reinterpret_cast<const uint4*>(P.c_words + P.c_off[p]);
-        uint4* dst = reinterpret_cast<uint4*>(prog);
-        for (uint32_t k = lane; k < P.c_size[p] / 4; k += 32) dst[k] = __ldg(src + k);
+        copy_program(P, p, prog, slot0 * 8, spare, lane);
         __syncwarp();
     }
     const uint64_t t_base = A.t0_dev ? *A.t0_dev + A.t0 : A.t0;
@@ -602,7 +697,8 @@ __global__ void __launch_bounds__(1024) k_cycles_cl(DevProg P, DevState S, Launc
             const uint32_t par = uint32_t(t & 1);
             const uint64_t* mc = mirror + (uint64_t)par * A.mirror_words;
             const uint32_t mn = smem_addr(mirror + (uint64_t)(par ^ 1) * A.mirror_words);
-            task_lane_op_res<DIGEST, PAIRS>(P, S, p, 0, t, pending, sl, prog, lane, slot_words - 1, mc, mn);
+            task_lane_op_res<DIGEST, PAIRS>(P, S, p, 0, t, pending, reinterpret_cast<char*>(smem), sl, prog, lane,
+                                            slot_words - 1, mc, mn);
         }
         const bool skip = (int32_t)blockIdx.x == A.skip_cta && c == 0;
         if (A.one_cluster && A.skip_cta < 0) {

@@ -79,7 +79,7 @@ int sm_count() {
 }
 
 // Dynamic shared memory a CTA of our kernels may use: the device's opt-in
-// limit less 1 KB for the kernels' static shared variables.
+// limit less 32 bytes for the kernels' static shared variables.
 size_t smem_limit() {
     int dev = 0, v = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -87,7 +87,7 @@ size_t smem_limit() {
         cudaGetLastError();
         return 220 * 1024;
     }
-    return size_t(v) - 1024;
+    return size_t(v) - 32;
 }
 
 // Shared memory a cluster CTA requests at least: more than half an SM's,
@@ -176,9 +176,9 @@ struct sim_batch {
     uint32_t n_inst = 0, I = 0;
     uint64_t seed = 0, cycle = 0;
     // program tables
-    DBuf s_ins, s_off, s_len, c_words, c_off, c_size, b_ins, b_off, b_len, mport_off, mport_id, mem_lg, mem_w, mem_base,
+    DBuf s_ins, s_off, s_len, e_words, c_off, c_size, e_tab, b_ins, b_off, b_len, mport_off, mport_id, mem_lg, mem_w, mem_base,
         in_w, reg_cls, reg_idx, mem_word_off, warp_proc, mir_off, mir_reg, warp_off, warp_slots,
-        proc_order;
+        warp_prog, proc_order;
     bool cluster = false;                   // cluster exchange kernel (k_cycles_cl)
     uint32_t mirror_off = 0;                // cluster CTA layout: mirror start (64-bit words)
     // state
@@ -195,6 +195,7 @@ struct sim_batch {
     int threads = 256, warps = 8, grid = 0, max_grid = 0;
     size_t smem = 0;
     uint32_t slot_words = 0, prog_words = 0, n_tasks = 0;
+    uint32_t replicas = 1;                  // warps per process (see LaunchArgs)
     uint32_t proc_major = 0;                // task order (see LaunchArgs)
     uint32_t wave_groups = 0;
     uint32_t cta_major = 0;
@@ -321,6 +322,7 @@ int sim_load_netlist(const void* text, size_t len, const sim_config* cfg, sim_ne
             rc = lower_clusters(h->nl, h->part, C, W, h->low, h->cplan, err, h->cfg.chain < 2);
             if (rc) return set_err(rc, err);
         }
+        encode_programs(h->low);
         h->layout = reg_layout(h->nl);
         const Netlist& nl = h->nl;
         h->mport_off.assign(1, 0);
@@ -543,6 +545,13 @@ uint32_t resident_words(const Lowered& L, uint32_t total_warps) {
     return uint32_t(std::min<uint64_t>(mx, 0xffffffffu));
 }
 
+// The operators of a resident program address the constant table and the
+// slots of a CTA with 16-bit byte offsets.  A value takes a slot (8 bytes) and
+// at least an instruction and a half (24) on chip, so no CTA whose programs fit
+// shared memory needs more slots than that, short of one that keeps nearly
+// every value it computes until the end.
+constexpr size_t kMaxSlotBytes = 65536;
+
 // Cluster exchange: one process per warp on the planned grid of clusters;
 // slots, resident program and the two mirror buffers in shared memory.
 int plan_launch_cluster(sim_batch* b) {
@@ -559,17 +568,25 @@ int plan_launch_cluster(sim_batch* b) {
     // pack each CTA's warps by their own process's slots (plus one spare) and
     // program; every area starts on 16 bytes (even slot words, programs in
     // multiples of 4 words)
-    std::vector<uint32_t> warp_off(cp.warp_proc.size(), 0), warp_slots(cp.warp_proc.size(), 0);
+    std::vector<uint32_t> warp_off(cp.warp_proc.size(), 0), warp_slots(cp.warp_proc.size(), 0),
+        warp_prog(cp.warp_proc.size(), 0);
     uint64_t max_cta = 0;
     for (uint32_t c = 0; c < cp.grid; c++) {
-        uint64_t off = 0;
+        uint64_t off = kTabWords;
         for (uint32_t w = 0; w < cp.W; w++) {
             const size_t i = size_t(c) * cp.W + w;
             const uint32_t p = cp.warp_proc[i];
             warp_off[i] = uint32_t(off);
             if (p == kNoProc) continue;
             warp_slots[i] = (L.s_slots[p] + 2) & ~1u;
-            off += warp_slots[i] + L.c_size[p] / 2;
+            off += warp_slots[i];
+        }
+        if (off * 8 > kMaxSlotBytes) return set_err(SIM_ERR_CAPACITY, "a cluster CTA needs too many value slots");
+        for (uint32_t w = 0; w < cp.W; w++) {
+            const size_t i = size_t(c) * cp.W + w;
+            const uint32_t p = cp.warp_proc[i];
+            warp_prog[i] = uint32_t(off);
+            if (p != kNoProc) off += L.c_size[p] / 2;
         }
         max_cta = std::max(max_cta, off);
     }
@@ -586,7 +603,10 @@ int plan_launch_cluster(sim_batch* b) {
         return set_err(SIM_ERR_CAPACITY, std::to_string(cp.grid / cp.C) + " clusters of " + std::to_string(cp.C) +
                                              " CTAs requested, " + std::to_string(n_clusters) + " can be resident");
     int rc;
-    if ((rc = upload(b->warp_off, warp_off, b->stream)) || (rc = upload(b->warp_slots, warp_slots, b->stream))) return rc;
+    if ((rc = upload(b->warp_off, warp_off, b->stream)) || (rc = upload(b->warp_slots, warp_slots, b->stream)) ||
+        (rc = upload(b->warp_prog, warp_prog, b->stream)))
+        return rc;
+    b->P.warp_prog = b->warp_prog.as<uint32_t>();
     b->P.warp_off = b->warp_off.as<uint32_t>();
     b->P.warp_slots = b->warp_slots.as<uint32_t>();
     CUDA_TRY(cudaStreamSynchronize(b->stream));
@@ -620,14 +640,15 @@ int plan_launch(sim_batch* b) {
     b->threads = warps * 32;
     b->prog_words = 0;
     int occ = 0;
+    b->replicas = 1;
     if (b->mode == SIM_MODE_LANE_OP) {
         // one process per warp when the grid allows it; re-plan with the
         // smaller grid if the resident programs lower occupancy
         uint32_t grid = (n_proc + warps - 1) / warps;
         for (int iter = 0; iter < 3; iter++) {
             uint32_t pw = (resident_words(L, grid * warps) + 3) & ~3u;
-            size_t smem = size_t(warps) * (slot_bytes + size_t(pw) * 4);
-            if (smem > smem_cap) break;
+            size_t smem = kTabWords * 8 + size_t(warps) * (slot_bytes + size_t(pw) * 4);
+            if (smem > smem_cap || kTabWords * 8 + size_t(warps) * slot_bytes > kMaxSlotBytes) break;
             CUDA_TRY(prepare_cycles_kernel(b->mode, smem));
             CUDA_TRY(occupancy_cycles(b->mode, b->threads, smem, &occ));
             if (occ < 1) break;
@@ -661,8 +682,8 @@ int upload_program(sim_batch* b) {
     std::vector<uint64_t> mem_base(nl.mem_lg.size());
     for (size_t m = 0; m < nl.mem_lg.size(); m++) mem_base[m] = h->mem_word_off[m] * b->I;
     if ((rc = upload(b->s_ins, L.s_ins, st)) || (rc = upload(b->s_off, L.s_off, st)) || (rc = upload(b->s_len, L.s_len, st)) ||
-        (rc = upload(b->c_words, L.c_words, st)) || (rc = upload(b->c_off, L.c_off, st)) ||
-        (rc = upload(b->c_size, L.c_size, st)) ||
+        (rc = upload(b->e_words, L.e_words, st)) || (rc = upload(b->c_off, L.c_off, st)) ||
+        (rc = upload(b->c_size, L.c_size, st)) || (rc = upload(b->e_tab, L.e_tab, st)) ||
         (rc = upload(b->b_ins, L.b_ins, st)) || (rc = upload(b->b_off, L.b_off, st)) || (rc = upload(b->b_len, L.b_len, st)) ||
         (rc = upload(b->mport_off, h->mport_off, st)) || (rc = upload(b->mport_id, h->mport_id, st)) ||
         (rc = upload(b->mem_lg, nl.mem_lg, st)) || (rc = upload(b->mem_w, nl.mem_w, st)) ||
@@ -681,9 +702,10 @@ int upload_program(sim_batch* b) {
     P.s_ins = b->s_ins.as<DIns>();
     P.s_off = b->s_off.as<uint32_t>();
     P.s_len = b->s_len.as<uint32_t>();
-    P.c_words = b->c_words.as<uint32_t>();
+    P.e_words = b->e_words.as<uint32_t>();
     P.c_off = b->c_off.as<uint32_t>();
     P.c_size = b->c_size.as<uint32_t>();
+    P.e_tab = b->e_tab.as<uint32_t>();
     P.b_ins = b->b_ins.as<DIns>();
     P.b_off = b->b_off.as<uint32_t>();
     P.b_len = b->b_len.as<uint32_t>();
@@ -887,6 +909,7 @@ LaunchArgs base_args(sim_batch* b) {
     A.warps_per_cta = uint32_t(b->warps);
     A.slot_words = b->slot_words;
     A.prog_words = b->prog_words;
+    A.replicas = b->replicas;
     A.n_tasks = b->n_tasks;
     A.group = b->mode == SIM_MODE_LANE_INST ? 32 : 1;
     A.proc_major = b->proc_major;
