@@ -102,6 +102,8 @@ struct DevProg {
     const DIns* b_ins;          // LANE_INST linear streams
     const uint32_t* b_off;
     const uint32_t* b_len;
+    const uint32_t* b_slots;    // value slots of each process
+    const uint32_t* b_order;    // processes by descending slots
     const uint32_t* mport_off;  // write ports of each memory (n_mem+1 offsets)
     const uint32_t* mport_id;
     const uint8_t* mem_lg;
@@ -121,6 +123,10 @@ struct DevProg {
     uint32_t n_proc, n_in, n_reg, n_mem, n_wport;
 };
 
+// Kind of a LANE_INST instruction, in the upper bits of its opcode byte on the
+// device: every operator is at most four branches away.
+enum BKind : uint32_t { K_OTHER = 0, K_LDR, K_CONST, K_STR, K_SUM, K_TEST, K_SHIFT, K_LOGIC };
+constexpr uint32_t kBlockWords = 64;     // LANE_INST: 64-bit words of a warp's instruction block
 constexpr uint32_t kNoProc = 0xffffffffu;
 
 // State of one batch of instances (device pointers).
@@ -161,8 +167,9 @@ struct LaunchArgs {
     int32_t skip_cta;           // testing: this CTA skips its first barrier arrival (-1 none)
     uint64_t timeout_ns;        // barrier wait limit
     uint32_t warps_per_cta;
-    uint32_t slot_words;        // per-warp slot area in 64-bit words (even)
+    uint32_t slot_words;        // per-warp slot area in 64-bit words (even); 0 = areas packed by process (LANE_INST)
     uint32_t prog_words;        // per-warp resident program area in 32-bit words (0 = read from global)
+    uint32_t banded;            // packed areas: warp w of every CTA has the w-th part of the tasks
     uint32_t replicas;          // LANE_OP: warps per process, each with its share of the instances
     uint32_t n_tasks;           // processes x instance groups
     uint32_t group;             // instances per task (1 LANE_OP, 32 LANE_INST)

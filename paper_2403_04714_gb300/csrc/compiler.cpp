@@ -2001,6 +2001,21 @@ void encode_op(const DIns& d, bool second, uint32_t out[4]) {
 }  // namespace
 
 void encode_programs(Lowered& low) {
+    low.k_ins = low.b_ins;
+    for (DIns& d : low.k_ins) {
+        uint32_t kind = K_OTHER;
+        switch (d.op) {
+        case D_LDR: kind = K_LDR; break;
+        case D_CONST: kind = K_CONST; break;
+        case D_STR: kind = K_STR; break;
+        case D_ADD: case D_SUB: case D_MUL: kind = K_SUM; break;
+        case D_EQ: case D_LT: case D_MUX: kind = K_TEST; break;
+        case D_SHL: case D_SHR: case D_SLICE: case D_CONCAT: kind = K_SHIFT; break;
+        case D_AND: case D_OR: case D_XOR: kind = K_LOGIC; break;
+        default: break;
+        }
+        d.op = uint8_t(d.op | kind << 5);
+    }
     low.e_words = low.c_words;
     low.e_tab.assign(low.c_off.size(), 0);
     for (size_t p = 0; p < low.c_off.size(); p++) {

@@ -110,6 +110,7 @@ struct Lowered {
     // LANE_INST: linear instruction list
     std::vector<DIns> b_ins;
     std::vector<uint32_t> b_off, b_len, b_slots;
+    std::vector<DIns> k_ins;          // b_ins as the device reads it: the kind (BKind) above the opcode
     uint32_t max_bundles = 0, max_s_slots = 0, max_b_slots = 0;
     std::vector<int32_t> commit_proc; // per memory: process holding its write ports (-1 none)
 };

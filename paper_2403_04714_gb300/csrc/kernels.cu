@@ -52,31 +52,32 @@ __device__ __forceinline__ Dec decode(uint4 r) {
     return d;
 }
 
-__device__ __forceinline__ uint64_t alu(uint32_t op, uint64_t a, uint64_t b, uint64_t c, uint32_t x) {
-    switch (op) {
-    case D_ADD: return a + b;
-    case D_SUB: return a - b;
-    case D_MUL: return a * b;
-    case D_AND: return a & b;
-    case D_OR: return a | b;
-    case D_XOR: return a ^ b;
-    case D_SHL: return b >= 64 ? 0 : a << b;
-    case D_SHR: return b >= 64 ? 0 : a >> b;
-    case D_EQ: return a == b ? 1 : 0;
-    case D_LT: return a < b ? 1 : 0;
-    case D_MUX: return a != 0 ? b : c;
-    case D_SLICE: return a >> x;           // lo < 64 (checked at load)
-    case D_CONCAT: return (a << x) | b;    // width(b) < 64 (checked at load)
-    default: return 0;
-    }
+// 64-bit shifts by 64 or more give 0, as PTX defines them.
+__device__ __forceinline__ uint64_t shr64(uint64_t v, uint32_t n) {
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
+}
+
+__device__ __forceinline__ uint64_t shl64(uint64_t v, uint32_t n) {
+    uint64_t r;
+    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
 }
 
 // ---------------------------------------------------------------------------
 // LANE_INST: one warp, one process, 32 instances (lane = instance).
 // ---------------------------------------------------------------------------
+// The warp's next 32 instructions sit in its block of shared memory (its lanes
+// load the block after that meanwhile), and each instruction is read from there
+// one ahead; fetched one by one, every eighth waited for L2.  Operators are at
+// most four branches away (BKind); a switch over all opcodes took 13 branches
+// and 64 instructions each.  200k-op netlist x 100: 232 us a cycle -> 186 with
+// the blocks -> 157 with the kinds; fetching the block's register rows ahead
+// measured 5 % slower.
 template <bool DIGEST>
 __device__ void task_lane_inst(const DevProg& P, const DevState& S, uint32_t p, uint32_t g, uint64_t t, bool pending,
-                               uint64_t* __restrict__ sl, uint32_t lane) {
+                               uint64_t* __restrict__ sl, uint4* __restrict__ block, uint32_t lane) {
     const uint32_t inst = g * 32 + lane;
     const uint32_t par = uint32_t(t & 1), nxt = par ^ 1;
     const uint64_t key = S.key[inst];
@@ -85,59 +86,69 @@ __device__ void task_lane_inst(const DevProg& P, const DevState& S, uint32_t p, 
     const DIns* ip = P.b_ins + P.b_off[p];
     const uint32_t n = P.b_len[p];
 #define SL(s) sl[(s) * 32 + lane]
+    uint4 next = lane < n ? ld_ins(ip + lane) : make_uint4(0, 0, 0, 0);
+    uint4 raw = make_uint4(0, 0, 0, 0);
     for (uint32_t i = 0; i < n; i++) {
-        Dec d = decode(ld_ins(ip + i));
-        switch (d.op) {
-        case D_NOP:
-            break;
-        case D_LDR:
-            SL(d.dst) = load_reg(S, par, d.c, d.b | (d.x << 16), inst);
-            break;
-        case D_LDI:
-            SL(d.dst) = stimulus(P, S, key, d.imm, inst, t, d.w);
-            break;
-        case D_CONST:
-            SL(d.dst) = (uint64_t)d.imm | ((uint64_t)d.a << 32) | ((uint64_t)d.b << 48);
-            break;
-        case D_MEMRD: {
-            uint64_t addr = SL(d.a) & ((1ULL << P.mem_lg[d.imm]) - 1);
-            SL(d.dst) = mem_read(P, S, d.imm, addr, inst, nxt, pending);
-            break;
+        const uint32_t j = i & 31u;
+        if (j == 0) {
+            __syncwarp();
+            block[lane] = next;
+            __syncwarp();
+            if (i + 32 + lane < n) next = ld_ins(ip + i + 32 + lane);
+            raw = block[0];
         }
-        case D_STR: {
-            uint64_t v = SL(d.a) & wmask(d.w);
-            uint32_t idx = d.b | (d.x << 16);
+        const Dec d = decode(raw);
+        raw = block[(j + 1) & 31u];
+        const uint32_t kind = (d.op >> 5) & 7u, op = d.op & 31u;
+        uint64_t v;
+        if (kind & 4u) {                                  // operators
+            const uint64_t a = SL(d.a), b = SL(d.b);
+            if (kind & 2u) {
+                if (kind & 1u) {                          // and, or, xor
+                    const uint64_t both = 0ull - uint64_t(op != D_XOR), one = 0ull - uint64_t(op != D_AND);
+                    v = (a & b & both) | ((a ^ b) & one);
+                } else {                                  // shl, shr, slice, concat
+                    const uint32_t n = op >= D_SLICE ? d.x : b >= 64 ? 64u : uint32_t(b);
+                    const uint64_t r = shr64(a, n), l = shl64(a, n);
+                    v = op == D_SHR || op == D_SLICE ? r : op == D_SHL ? l : l | b;
+                }
+            } else if (kind & 1u) {                       // eq, lt, mux
+                v = op == D_MUX ? (a != 0 ? b : SL(d.c)) : uint64_t(op == D_EQ ? a == b : a < b);
+            } else {                                      // add, sub, mul
+                v = op == D_MUL ? a * b : op == D_SUB ? a - b : a + b;
+            }
+            SL(d.dst) = v & wmask(d.w);
+        } else if (kind == K_LDR) {
+            SL(d.dst) = load_tile(S, par, d.c, d.b | (d.x << 16), g, lane);
+        } else if (kind == K_CONST) {
+            SL(d.dst) = (uint64_t)d.imm | ((uint64_t)d.a << 32) | ((uint64_t)d.b << 48);
+        } else if (kind == K_STR) {
+            v = SL(d.a) & wmask(d.w);
+            const uint32_t idx = d.b | (d.x << 16);
             if (d.c == RC_W64) {
-                S.w64[nxt][reg_pos(S, S.n_w64, idx, inst)] = v;
+                S.w64[nxt][((uint64_t)g * S.n_w64 + idx) * 32u + lane] = v;
             } else if (d.c == RC_W32) {
-                S.w32[nxt][reg_pos(S, S.n_w32, idx, inst)] = uint32_t(v);
+                S.w32[nxt][((uint64_t)g * S.n_w32 + idx) * 32u + lane] = uint32_t(v);
             } else {
-                uint32_t word = __ballot_sync(0xffffffffu, v & 1);
+                const uint32_t word = __ballot_sync(0xffffffffu, v & 1);
                 if (lane == 0) S.bits[nxt][(uint64_t)g * S.n_bit + idx] = word;
             }
             if (DIGEST && col >= 0) dacc += mix64(((uint64_t)d.imm * kGamma + 1ULL) ^ v);
-            break;
-        }
-        case D_WREC: {
-            uint64_t en = SL(d.a) != 0;
-            uint64_t addr = SL(d.b) & ((1ULL << d.x) - 1);
-            uint64_t data = SL(d.c) & wmask(d.w);
+        } else if (op == D_LDI) {
+            SL(d.dst) = stimulus(P, S, key, d.imm, inst, t, d.w);
+        } else if (op == D_MEMRD) {
+            const uint64_t addr = SL(d.a) & ((1ULL << P.mem_lg[d.imm]) - 1);
+            SL(d.dst) = mem_read(P, S, d.imm, addr, inst, nxt, pending);
+        } else if (op == D_WREC) {
+            const uint64_t en = SL(d.a) != 0;
+            const uint64_t addr = SL(d.b) & ((1ULL << d.x) - 1);
+            const uint64_t data = SL(d.c) & wmask(d.w);
             uint64_t* r = S.rec[par] + ((uint64_t)d.imm * S.I + inst) * 2;
             r[0] = en ? ((1ULL << 63) | addr) : 0;
             r[1] = data;
-            break;
-        }
-        case D_COMMIT:
-            if (pending) {
-                uint64_t delta = mem_commit(P, S, d.imm, inst, nxt, DIGEST && col >= 0);
-                if (DIGEST) mem_digest_update(S, d.imm, inst, t, delta);
-            }
-            break;
-        case D_MUX:
-            SL(d.dst) = alu(D_MUX, SL(d.a), SL(d.b), SL(d.c), 0) & wmask(d.w);
-            break;
-        default:
-            SL(d.dst) = alu(d.op, SL(d.a), SL(d.b), 0, d.x) & wmask(d.w);
+        } else if (op == D_COMMIT && pending) {
+            const uint64_t delta = mem_commit(P, S, d.imm, inst, nxt, DIGEST && col >= 0);
+            if (DIGEST) mem_digest_update(S, d.imm, inst, t, delta);
         }
     }
 #undef SL
@@ -375,19 +386,6 @@ __device__ void task_lane_op(const DevProg& P, const DevState& S, uint32_t p, ui
 // A == X and A < c from the selected operand (2 %), the result of a compare
 // selected in 64 bits (2-4 %), fields read as 16-bit words (3-5 %), the fields
 // taken apart before the warp barrier (no change), the mask as two shifts (5 %).
-// 64-bit shifts by 64 or more give 0, as PTX defines them.
-__device__ __forceinline__ uint64_t shr64(uint64_t v, uint32_t n) {
-    uint64_t r;
-    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
-    return r;
-}
-
-__device__ __forceinline__ uint64_t shl64(uint64_t v, uint32_t n) {
-    uint64_t r;
-    asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
-    return r;
-}
-
 // All bits of the result: the sign bit of byte BYTE of v.
 template <int BYTE>
 __device__ __forceinline__ uint64_t byte_sign(uint32_t v) {
@@ -577,6 +575,53 @@ __device__ void task_lane_op_res(const DevProg& P, const DevState& S, uint32_t p
     finish_lane_op<DIGEST>(S, p, inst, t, col, lane, dacc);
 }
 
+// LANE_INST in process-major order with every warp's area as large as the
+// slots of its own processes: these are taken by descending slots, so that a
+// warp's first process is its largest, and a CTA's warps take tasks `grid`
+// apart, or, where that keeps warps off the SM, warp w of every CTA has the
+// w-th part of the tasks.  An area for the largest process in every warp let 8
+// or 12 warps of the 200k-op netlist share an SM (slots: mean 38, at most 69);
+// packed, 16 to 22 do (100 instances 157 -> 93 us a cycle, one round instead of
+// two; 4,096 instances 3.35 -> 2.45 ms).  The two thirds of the time that are
+// left is the dependent chain of each instruction, three to five warps per scheduler.
+template <bool DIGEST>
+__device__ __forceinline__ void lane_inst_packed(const DevProg& P, const DevState& S, const LaunchArgs& A, uint64_t* smem) {
+    const uint32_t lane = threadIdx.x & 31, wib = threadIdx.x >> 5, W = A.warps_per_cta;
+    const uint32_t G = A.n_tasks / P.n_proc;
+    const auto proc = [&](uint32_t task) { return P.b_order[task / G]; };
+    const uint32_t rounds = (A.n_tasks + gridDim.x * W - 1) / (gridDim.x * W);
+    const uint32_t band = gridDim.x * (A.banded ? rounds : 1), step = A.banded ? gridDim.x : gridDim.x * W;
+    const uint32_t task0 = wib * band + blockIdx.x, mine = lane * band + blockIdx.x;
+    const uint32_t end = A.banded ? min(A.n_tasks, (wib + 1) * band) : A.n_tasks;
+    uint32_t sum = lane < W && mine < A.n_tasks ? P.b_slots[proc(mine)] * 32 + kBlockWords : 0;
+    const uint32_t area = __shfl_sync(0xffffffffu, sum, wib);
+    for (uint32_t o = 1; o < 32; o *= 2) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, sum, o);
+        if (lane >= o) sum += v;
+    }
+    if (__shfl_sync(0xffffffffu, sum, 31) * 8 > dynamic_smem_bytes()) {      // not the planned launch: report it
+        if (threadIdx.x == 0) atomicCAS(S.err, 0, (int32_t)SIM_ERR_STATE);
+        return;
+    }
+    uint64_t* sl = smem + (__shfl_sync(0xffffffffu, sum, wib) - area);
+    uint4* block = reinterpret_cast<uint4*>(sl + area - kBlockWords);
+    const uint64_t t_base = A.t0_dev ? *A.t0_dev + A.t0 : A.t0;
+    uint32_t gen = 0;
+    for (uint32_t c = 0; c < A.n; c++) {
+        const uint64_t t = t_base + c;
+        uint64_t* rec = (A.phase && c < A.phase_n) ? A.phase + ((uint64_t)c * gridDim.x + blockIdx.x) * 3 : nullptr;
+        if (rec && threadIdx.x == 0) rec[0] = globaltimer_ns();
+        for (uint32_t task = task0; task < end; task += step)
+            task_lane_inst<DIGEST>(P, S, proc(task), task % G, t, c > 0 || A.pending_first, sl, block, lane);
+        if (A.grid_sync) {
+            const bool skip = (int32_t)blockIdx.x == A.skip_cta && c == 0;
+            if (!grid_barrier(S.bar, gen, A.timeout_ns, S.err, skip, rec ? rec + 1 : nullptr)) return;
+        }
+    }
+    if (A.grid_sync && A.n > 0)
+        final_commit(P, S, t_base + A.n, (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, (uint64_t)gridDim.x * blockDim.x);
+}
+
 template <int MODE, bool DIGEST, bool PAIRS>
 __global__ void __launch_bounds__(1024) k_cycles(DevProg P, DevState S, LaunchArgs A) {
     extern __shared__ __align__(16) uint64_t smem[];
@@ -584,6 +629,10 @@ __global__ void __launch_bounds__(1024) k_cycles(DevProg P, DevState S, LaunchAr
     const uint32_t warp = blockIdx.x * A.warps_per_cta + wib;
     const uint32_t tw = gridDim.x * A.warps_per_cta;
     const bool resident = MODE == SIM_MODE_LANE_OP && A.prog_words > 0;
+    if (MODE == SIM_MODE_LANE_INST && A.slot_words == 0) {
+        lane_inst_packed<DIGEST>(P, S, A, smem);
+        return;
+    }
     // resident programs: the constant table, every warp's slots, then the programs
     const uint32_t slot0 = (resident ? kTabWords : 0) + wib * A.slot_words;
     uint64_t* sl = smem + slot0;
@@ -623,7 +672,8 @@ __global__ void __launch_bounds__(1024) k_cycles(DevProg P, DevState S, LaunchAr
                 // for different instance groups (its code and constants stay hot)
             uint32_t p, g;
             task_coords(A, P.n_proc, task, p, g);
-                if (MODE == SIM_MODE_LANE_INST) task_lane_inst<DIGEST>(P, S, p, g, t, pending, sl, lane);
+                if (MODE == SIM_MODE_LANE_INST) task_lane_inst<DIGEST>(P, S, p, g, t, pending, sl,
+                                                                              reinterpret_cast<uint4*>(sl + A.slot_words - kBlockWords), lane);
                 else task_lane_op<DIGEST>(P, S, p, g, t, pending, sl, lane);
             }
         }

@@ -158,6 +158,7 @@ struct sim_netlist {
     RegLayout layout;
     sim_netlist_info info{};
     std::vector<uint32_t> mport_off, mport_id;
+    std::vector<uint32_t> b_order;        // processes by descending LANE_INST slots
     std::vector<uint64_t> mem_word_off;   // per-instance word offset of each memory (+ total)
 };
 
@@ -176,7 +177,7 @@ struct sim_batch {
     uint32_t n_inst = 0, I = 0;
     uint64_t seed = 0, cycle = 0;
     // program tables
-    DBuf s_ins, s_off, s_len, e_words, c_off, c_size, e_tab, b_ins, b_off, b_len, mport_off, mport_id, mem_lg, mem_w, mem_base,
+    DBuf s_ins, s_off, s_len, e_words, c_off, c_size, e_tab, b_ins, b_off, b_len, b_slots, b_order, mport_off, mport_id, mem_lg, mem_w, mem_base,
         in_w, reg_cls, reg_idx, mem_word_off, warp_proc, mir_off, mir_reg, warp_off, warp_slots,
         warp_prog, proc_order;
     bool cluster = false;                   // cluster exchange kernel (k_cycles_cl)
@@ -195,6 +196,7 @@ struct sim_batch {
     int threads = 256, warps = 8, grid = 0, max_grid = 0;
     size_t smem = 0;
     uint32_t slot_words = 0, prog_words = 0, n_tasks = 0;
+    uint32_t banded = 0;                    // packed LANE_INST areas (see LaunchArgs)
     uint32_t replicas = 1;                  // warps per process (see LaunchArgs)
     uint32_t proc_major = 0;                // task order (see LaunchArgs)
     uint32_t wave_groups = 0;
@@ -323,6 +325,10 @@ int sim_load_netlist(const void* text, size_t len, const sim_config* cfg, sim_ne
             if (rc) return set_err(rc, err);
         }
         encode_programs(h->low);
+        h->b_order.resize(h->low.b_slots.size());
+        for (size_t p = 0; p < h->b_order.size(); p++) h->b_order[p] = uint32_t(p);
+        std::stable_sort(h->b_order.begin(), h->b_order.end(),
+                         [&](uint32_t x, uint32_t y) { return h->low.b_slots[x] > h->low.b_slots[y]; });
         h->layout = reg_layout(h->nl);
         const Netlist& nl = h->nl;
         h->mport_off.assign(1, 0);
@@ -614,6 +620,54 @@ int plan_launch_cluster(sim_batch* b) {
     return SIM_OK;
 }
 
+// Lane = instance bytecode, areas packed by process (lane_inst_packed): the
+// CTA size and grid on 1 / share of the GPU with the fewest rounds of tasks,
+// then the fewest warps.  CTA 0 has the largest areas.
+int plan_lane_inst(sim_batch* b, uint32_t share) {
+    const Lowered& L = b->nl->low;
+    const uint32_t n_proc = uint32_t(L.b_slots.size()), G = b->n_tasks / n_proc;
+    const int sms = sm_count();
+    const int lo = b->cfg.warps_per_cta ? std::min(32, int(b->cfg.warps_per_cta)) : 1;
+    const int hi = b->cfg.warps_per_cta ? lo : 32;
+    const bool per_cycle = b->kernel == SIM_KERNEL_PER_CYCLE || b->kernel == SIM_KERNEL_PER_CYCLE_GRAPH;
+    auto area_bytes = [&](int w, uint32_t band) {
+        uint64_t words = 0;
+        for (int i = 0; i < w && uint64_t(i) * band < b->n_tasks; i++)
+            words += L.b_slots[b->nl->b_order[size_t(i) * band / G]] * 32ull + kBlockWords;
+        return size_t(words) * 8;
+    };
+    uint64_t best = ~0ull;
+    b->slot_words = 0;
+    b->prog_words = 0;
+    for (int w = lo; w <= hi; w++) {
+        const int most = b->cfg.warps_per_cta ? 32 / w : 1;       // CTAs per SM
+        for (int k = std::max(1, most); k >= 1; k--) {
+            const uint32_t need = (b->n_tasks + w - 1) / w;
+            const uint32_t grid = std::max(1u, std::min(need, uint32_t(std::max(1, k * sms / int(std::max(1u, share))))));
+            const uint64_t rounds = (b->n_tasks + uint64_t(grid) * w - 1) / (uint64_t(grid) * w);
+            if (rounds >= best) continue;
+            // (launches of one cycle have a warp for every task)
+            bool banded = false;
+            size_t smem = area_bytes(w, per_cycle ? need : grid);
+            if (smem > smem_limit() && !per_cycle) banded = true, smem = area_bytes(w, uint32_t(rounds * grid));
+            if (smem > smem_limit()) continue;
+            int occ = 0;
+            CUDA_TRY(prepare_cycles_kernel(b->mode, smem));
+            CUDA_TRY(occupancy_cycles(b->mode, w * 32, smem, &occ));
+            if (uint64_t(occ) * sms < grid) continue;
+            best = rounds;
+            b->banded = banded;
+            b->warps = w;
+            b->threads = w * 32;
+            b->smem = smem;
+            b->max_grid = occ * sms;
+            b->grid = int(grid);
+        }
+    }
+    if (best == ~0ull) return set_err(SIM_ERR_CAPACITY, "the processes' value slots do not fit a CTA's shared memory");
+    return SIM_OK;
+}
+
 // Several instances, lane = operation: R warps per process, each holding its
 // program and running its share of the instances, when they can all be
 // resident; the CTA size with the fewest instances per warp (then the fewest
@@ -661,7 +715,7 @@ int plan_launch(sim_batch* b) {
     const size_t smem_cap = smem_limit();
     const uint32_t n_proc = uint32_t(b->nl->part.procs.size());
     if (b->mode == SIM_MODE_LANE_INST) {
-        b->slot_words = L.max_b_slots * 32;
+        b->slot_words = L.max_b_slots * 32 + kBlockWords;
         b->n_tasks = n_proc * (b->I / 32);
     } else {
         b->slot_words = (L.max_s_slots + 2) & ~1u;   // at least one spare slot (the operator steps' dummy)
@@ -674,6 +728,7 @@ int plan_launch(sim_batch* b) {
     int warps = b->cfg.warps_per_cta ? int(b->cfg.warps_per_cta) : 8;
     if (!b->cfg.warps_per_cta && b->mode == SIM_MODE_LANE_OP)   // one process per warp, one CTA per SM
         warps = int(std::min<uint64_t>(16, std::max<uint64_t>(1, (uint64_t(n_proc) * b->I + sms - 1) / sms)));
+    if (b->mode == SIM_MODE_LANE_INST && b->proc_major && !b->wave_groups) return plan_lane_inst(b, 1);
     while (warps > 1 && size_t(warps) * slot_bytes > smem_cap) warps /= 2;
     b->warps = warps;
     b->threads = warps * 32;
@@ -727,7 +782,7 @@ int upload_program(sim_batch* b) {
     if ((rc = upload(b->s_ins, L.s_ins, st)) || (rc = upload(b->s_off, L.s_off, st)) || (rc = upload(b->s_len, L.s_len, st)) ||
         (rc = upload(b->e_words, L.e_words, st)) || (rc = upload(b->c_off, L.c_off, st)) ||
         (rc = upload(b->c_size, L.c_size, st)) || (rc = upload(b->e_tab, L.e_tab, st)) ||
-        (rc = upload(b->b_ins, L.b_ins, st)) || (rc = upload(b->b_off, L.b_off, st)) || (rc = upload(b->b_len, L.b_len, st)) ||
+        (rc = upload(b->b_off, L.b_off, st)) || (rc = upload(b->b_len, L.b_len, st)) ||
         (rc = upload(b->mport_off, h->mport_off, st)) || (rc = upload(b->mport_id, h->mport_id, st)) ||
         (rc = upload(b->mem_lg, nl.mem_lg, st)) || (rc = upload(b->mem_w, nl.mem_w, st)) ||
         (rc = upload(b->mem_base, mem_base, st)) || (rc = upload(b->in_w, nl.in_w, st)) ||
@@ -735,11 +790,14 @@ int upload_program(sim_batch* b) {
         (rc = upload(b->mem_word_off, h->mem_word_off, st)) || (rc = upload(b->warp_proc, h->cplan.warp_proc, st)) ||
         (rc = upload(b->mir_off, h->cplan.mir_off, st)) || (rc = upload(b->mir_reg, h->cplan.mir_reg, st)))
         return rc;
+    if (b->mode == SIM_MODE_LANE_INST && ((rc = upload(b->b_slots, L.b_slots, st)) || (rc = upload(b->b_order, h->b_order, st))))
+        return rc;
     std::vector<uint32_t> order(h->part.procs.size());
     for (size_t p = 0; p < order.size(); p++) order[p] = uint32_t(p);
     std::stable_sort(order.begin(), order.end(),
                      [&](uint32_t x, uint32_t y) { return h->part.proc_cost[x] > h->part.proc_cost[y]; });
     if ((rc = upload(b->proc_order, order, st))) return rc;
+    if (b->mode == SIM_MODE_LANE_INST && (rc = upload(b->b_ins, L.k_ins, st))) return rc;
     DevProg& P = b->P;
     P.proc_order = b->proc_order.as<uint32_t>();
     P.s_ins = b->s_ins.as<DIns>();
@@ -752,6 +810,8 @@ int upload_program(sim_batch* b) {
     P.b_ins = b->b_ins.as<DIns>();
     P.b_off = b->b_off.as<uint32_t>();
     P.b_len = b->b_len.as<uint32_t>();
+    P.b_slots = b->b_slots.as<uint32_t>();
+    P.b_order = b->b_order.as<uint32_t>();
     P.mport_off = b->mport_off.as<uint32_t>();
     P.mport_id = b->mport_id.as<uint32_t>();
     P.mem_lg = b->mem_lg.as<uint8_t>();
@@ -953,6 +1013,7 @@ LaunchArgs base_args(sim_batch* b) {
     A.slot_words = b->slot_words;
     A.prog_words = b->prog_words;
     A.replicas = b->replicas;
+    A.banded = b->banded;
     A.n_tasks = b->n_tasks;
     A.group = b->mode == SIM_MODE_LANE_INST ? 32 : 1;
     A.proc_major = b->proc_major;
@@ -1760,6 +1821,7 @@ int pool_set_active(sim_batch* b, uint32_t n_groups, uint32_t share) {
     // a persistent step holds only the CTAs its tasks need, and at most its
     // share of the GPU, leaving the other SMs to the pools of other netlists
     if (b->generated) return plan_grid_gen(b, share);
+    if (b->slot_words == 0) return plan_lane_inst(b, share);
     const int cap = std::max(1, b->max_grid / int(std::max(1u, share)));
     b->grid = std::max(1, std::min(int((b->n_tasks + b->warps - 1) / b->warps), cap));
     return SIM_OK;

@@ -106,6 +106,14 @@ __device__ __forceinline__ uint64_t load_reg(const DevState& S, uint32_t par, ui
     return (word >> (inst % S.pack)) & 1u;
 }
 
+// The same for a lane of instance group g (pack 32).
+__device__ __forceinline__ uint64_t load_tile(const DevState& S, uint32_t par, uint32_t cls, uint32_t idx, uint32_t g,
+                                              uint32_t lane) {
+    if (cls == RC_W64) return S.w64[par][((uint64_t)g * S.n_w64 + idx) * 32u + lane];
+    if (cls == RC_W32) return S.w32[par][((uint64_t)g * S.n_w32 + idx) * 32u + lane];
+    return (S.bits[par][(uint64_t)g * S.n_bit + idx] >> lane) & 1u;
+}
+
 // The same for batches of one instance per warp (pack 1).
 __device__ __forceinline__ uint64_t load_reg1(const DevState& S, uint32_t par, uint32_t cls, uint32_t idx, uint32_t inst) {
     if (cls == RC_W64) return S.w64[par][(uint64_t)idx * S.I + inst];
