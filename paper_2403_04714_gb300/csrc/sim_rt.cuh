@@ -49,6 +49,10 @@ __device__ __forceinline__ void red_release_add(unsigned long long* p, unsigned 
 // by __syncthreads, become visible to every CTA that acquires the count) and
 // then polls the counter with acquire loads; nobody has to reset a counter or
 // publish a generation word, so the last arrival releases everyone directly.
+// The error word and the clock are read after every sixteenth poll: after each
+// one they doubled the time between polls (2k-op netlist 3.83 -> 3.76 us a
+// cycle, 200k-op netlist 9.11 -> 9.05).  A flag per CTA, polled by every other
+// CTA's warp, measured 3 us slower a cycle.
 // Every wait is bounded: past `timeout_ns`, or once another CTA has recorded
 // an error, the CTA records SIM_ERR_TIMEOUT (first error wins) and returns
 // false.  With `rec` set, thread 0 stores the time the whole CTA arrived
@@ -63,10 +67,13 @@ static __device__ bool grid_barrier(uint32_t* bar, uint32_t& gen, uint64_t timeo
         unsigned long long* count = reinterpret_cast<unsigned long long*>(bar);
         const unsigned long long target = (unsigned long long)(gen + 1) * gridDim.x;
         if (!skip) red_release_add(count, 1ull);
-        const uint64_t start = globaltimer_ns();
-        while (ld_acquire_u64(count) < target) {
+        uint64_t start = 0;
+        for (uint32_t polls = 1; ld_acquire_u64(count) < target; polls++) {
+            if (polls & 15u) continue;
+            const uint64_t now = globaltimer_ns();
+            if (!start) start = now;
             if (ld_volatile(err) != 0) { ok = 0; break; }
-            if (globaltimer_ns() - start > timeout_ns) {
+            if (now - start > timeout_ns) {
                 atomicCAS(err, 0, (int32_t)SIM_ERR_TIMEOUT);
                 ok = 0;
                 break;
