@@ -827,6 +827,15 @@ __global__ void k_reset_slots(DevProg P, DevState S, uint32_t par, uint32_t lo, 
         const_cast<uint8_t*>(S.hold_flag)[(e / n) * S.I + lo + e % n] = 0;
 }
 
+// Read-back of one instance into pinned host memory: every register in register
+// order (mem < 0) or the words of one memory, after the launch's error word.
+__global__ void k_read(DevProg P, DevState S, uint32_t par, uint32_t inst, int32_t mem, uint32_t n, uint64_t* out) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) out[0] = uint64_t(uint32_t(*S.err));
+    if (i >= n) return;
+    out[1 + i] = mem < 0 ? load_reg(S, par, P.reg_cls[i], P.reg_idx[i], inst) : S.mem[P.mem_base[mem] + (uint64_t)i * S.I + inst];
+}
+
 // Registers of buffer `par` between the kernels' tiles and the checkpoint's
 // order ([register][instance], 1-bit registers [register][group word]), which
 // uses buffer par ^ 1: its contents are dead between steps.
@@ -1012,6 +1021,12 @@ cudaError_t launch_reset_slots(cudaStream_t st, const DevProg& P, const DevState
                                uint64_t mem_words, const uint64_t* mem_init_dig, uint64_t rom_init_dig) {
     k_reset_slots<<<256, 256, 0, st>>>(P, S, par, lo, n, reg_init, mem_image, mem_word_off, mem_words, mem_init_dig,
                                        rom_init_dig);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_read(cudaStream_t st, const DevProg& P, const DevState& S, uint32_t par, uint32_t inst, int32_t mem,
+                        uint32_t n, uint64_t* out) {
+    k_read<<<std::max(1u, (n + 255) / 256), 256, 0, st>>>(P, S, par, inst, mem, n, out);
     return cudaGetLastError();
 }
 

@@ -30,6 +30,8 @@ cudaError_t launch_cycles_cl(bool digest, int grid, int threads, size_t smem, ui
                              const DevProg& P, const DevState& S, const LaunchArgs& A);
 cudaError_t launch_advance(cudaStream_t st, uint64_t* t0_dev, uint64_t n);
 cudaError_t launch_stim(cudaStream_t st, const DevProg& P, const DevState& S, uint64_t t, const uint64_t* t0_dev);
+cudaError_t launch_read(cudaStream_t st, const DevProg& P, const DevState& S, uint32_t par, uint32_t inst, int32_t mem,
+                        uint32_t n, uint64_t* out);
 cudaError_t launch_retile(cudaStream_t st, const DevState& S, uint32_t par, bool to_tiles);
 cudaError_t launch_set_u64(cudaStream_t st, uint64_t* p, uint64_t v);
 cudaError_t launch_state_digest(cudaStream_t st, const DevProg& P, const DevState& S, uint32_t par,
@@ -138,6 +140,51 @@ int upload(DBuf& b, const std::vector<T>& v, cudaStream_t st) {
 
 }  // namespace
 
+// Pinned host buffers of read-backs, shared by the batches of the process: a
+// call takes one for its duration (any thread, any stream), at most
+// kStageBuffers are kept, and the last batch's end frees them.
+namespace {
+constexpr size_t kStageBytes = 1 << 20;
+constexpr size_t kStageBuffers = 4;
+std::mutex g_stage_mu;
+std::vector<void*> g_stage_free;
+size_t g_stage_users = 0;
+
+void stage_retain() {
+    std::lock_guard<std::mutex> g(g_stage_mu);
+    g_stage_users++;
+}
+void stage_release() {
+    std::lock_guard<std::mutex> g(g_stage_mu);
+    if (--g_stage_users) return;
+    for (void* p : g_stage_free) cudaFreeHost(p);
+    g_stage_free.clear();
+}
+struct Stage {
+    uint64_t* p = nullptr;
+    int take() {
+        {
+            std::lock_guard<std::mutex> g(g_stage_mu);
+            if (!g_stage_free.empty()) {
+                p = static_cast<uint64_t*>(g_stage_free.back());
+                g_stage_free.pop_back();
+                return SIM_OK;
+            }
+        }
+        void* v = nullptr;
+        CUDA_TRY(cudaHostAlloc(&v, kStageBytes, cudaHostAllocPortable | cudaHostAllocMapped));
+        p = static_cast<uint64_t*>(v);
+        return SIM_OK;
+    }
+    ~Stage() {
+        if (!p) return;
+        std::lock_guard<std::mutex> g(g_stage_mu);
+        if (g_stage_free.size() < kStageBuffers) g_stage_free.push_back(p);
+        else cudaFreeHost(p);
+    }
+};
+}  // namespace
+
 struct sim_netlist {
     sim_config cfg;
     // generated-CUDA lowering, per lane mapping (built on first use)
@@ -159,6 +206,7 @@ struct sim_netlist {
     sim_netlist_info info{};
     std::vector<uint32_t> mport_off, mport_id;
     std::vector<uint32_t> b_order;        // processes by descending LANE_INST slots
+    std::vector<uint32_t> g_order;        // processes by descending cost
     std::vector<uint64_t> mem_word_off;   // per-instance word offset of each memory (+ total)
 };
 
@@ -221,7 +269,9 @@ struct sim_batch {
     DevState graph_state{};               // state descriptor captured in the graph
     bool own_stream = false;
     int device = 0;                        // device current when the batch was created
+    sim_batch() { stage_retain(); }
     ~sim_batch() {
+        stage_release();
         if (pool) rtl::pool_extra_free(pool);
         if (graph) cudaGraphExecDestroy(graph);
         if (pgraph) cudaGraphExecDestroy(pgraph);
@@ -325,10 +375,14 @@ int sim_load_netlist(const void* text, size_t len, const sim_config* cfg, sim_ne
             if (rc) return set_err(rc, err);
         }
         encode_programs(h->low);
-        h->b_order.resize(h->low.b_slots.size());
-        for (size_t p = 0; p < h->b_order.size(); p++) h->b_order[p] = uint32_t(p);
-        std::stable_sort(h->b_order.begin(), h->b_order.end(),
-                         [&](uint32_t x, uint32_t y) { return h->low.b_slots[x] > h->low.b_slots[y]; });
+        auto descending = [](const auto& key) {
+            std::vector<uint32_t> v(key.size());
+            for (size_t p = 0; p < v.size(); p++) v[p] = uint32_t(p);
+            std::stable_sort(v.begin(), v.end(), [&](uint32_t x, uint32_t y) { return key[x] > key[y]; });
+            return v;
+        };
+        h->b_order = descending(h->low.b_slots);
+        h->g_order = descending(h->part.proc_cost);
         h->layout = reg_layout(h->nl);
         const Netlist& nl = h->nl;
         h->mport_off.assign(1, 0);
@@ -779,25 +833,26 @@ int upload_program(sim_batch* b) {
     int rc;
     std::vector<uint64_t> mem_base(nl.mem_lg.size());
     for (size_t m = 0; m < nl.mem_lg.size(); m++) mem_base[m] = h->mem_word_off[m] * b->I;
-    if ((rc = upload(b->s_ins, L.s_ins, st)) || (rc = upload(b->s_off, L.s_off, st)) || (rc = upload(b->s_len, L.s_len, st)) ||
-        (rc = upload(b->e_words, L.e_words, st)) || (rc = upload(b->c_off, L.c_off, st)) ||
-        (rc = upload(b->c_size, L.c_size, st)) || (rc = upload(b->e_tab, L.e_tab, st)) ||
-        (rc = upload(b->b_off, L.b_off, st)) || (rc = upload(b->b_len, L.b_len, st)) ||
-        (rc = upload(b->mport_off, h->mport_off, st)) || (rc = upload(b->mport_id, h->mport_id, st)) ||
+    // the program tables of this batch's kernels only (generated code has none)
+    const bool gen = b->cfg.lowering == SIM_LOWER_GENERATED && !b->cfg.cluster_size;
+    if (gen && (rc = upload(b->proc_order, h->g_order, st))) return rc;
+    if (!gen && b->mode == SIM_MODE_LANE_OP &&
+        ((rc = upload(b->s_ins, L.s_ins, st)) || (rc = upload(b->s_off, L.s_off, st)) || (rc = upload(b->s_len, L.s_len, st)) ||
+         (rc = upload(b->e_words, L.e_words, st)) || (rc = upload(b->c_off, L.c_off, st)) ||
+         (rc = upload(b->c_size, L.c_size, st)) || (rc = upload(b->e_tab, L.e_tab, st)) ||
+         (rc = upload(b->warp_proc, h->cplan.warp_proc, st)) || (rc = upload(b->mir_off, h->cplan.mir_off, st)) ||
+         (rc = upload(b->mir_reg, h->cplan.mir_reg, st))))
+        return rc;
+    if (!gen && b->mode == SIM_MODE_LANE_INST &&
+        ((rc = upload(b->b_ins, L.k_ins, st)) || (rc = upload(b->b_off, L.b_off, st)) || (rc = upload(b->b_len, L.b_len, st)) ||
+         (rc = upload(b->b_slots, L.b_slots, st)) || (rc = upload(b->b_order, h->b_order, st))))
+        return rc;
+    if ((rc = upload(b->mport_off, h->mport_off, st)) || (rc = upload(b->mport_id, h->mport_id, st)) ||
         (rc = upload(b->mem_lg, nl.mem_lg, st)) || (rc = upload(b->mem_w, nl.mem_w, st)) ||
         (rc = upload(b->mem_base, mem_base, st)) || (rc = upload(b->in_w, nl.in_w, st)) ||
         (rc = upload(b->reg_cls, h->layout.cls, st)) || (rc = upload(b->reg_idx, h->layout.idx, st)) ||
-        (rc = upload(b->mem_word_off, h->mem_word_off, st)) || (rc = upload(b->warp_proc, h->cplan.warp_proc, st)) ||
-        (rc = upload(b->mir_off, h->cplan.mir_off, st)) || (rc = upload(b->mir_reg, h->cplan.mir_reg, st)))
+        (rc = upload(b->mem_word_off, h->mem_word_off, st)))
         return rc;
-    if (b->mode == SIM_MODE_LANE_INST && ((rc = upload(b->b_slots, L.b_slots, st)) || (rc = upload(b->b_order, h->b_order, st))))
-        return rc;
-    std::vector<uint32_t> order(h->part.procs.size());
-    for (size_t p = 0; p < order.size(); p++) order[p] = uint32_t(p);
-    std::stable_sort(order.begin(), order.end(),
-                     [&](uint32_t x, uint32_t y) { return h->part.proc_cost[x] > h->part.proc_cost[y]; });
-    if ((rc = upload(b->proc_order, order, st))) return rc;
-    if (b->mode == SIM_MODE_LANE_INST && (rc = upload(b->b_ins, L.k_ins, st))) return rc;
     DevProg& P = b->P;
     P.proc_order = b->proc_order.as<uint32_t>();
     P.s_ins = b->s_ins.as<DIns>();
@@ -873,19 +928,23 @@ int init_state(sim_batch* b) {
                 std::fill_n(bitw.begin() + size_t(ix) * words, words, word);
             }
         }
-        // the tile from the host, then copies of it on the device, doubling
-        auto spread = [&](void* dst, const void* tile, size_t bytes) -> int {
+        // up to 1 MB of tiles from the host, then copies of them on the device, doubling
+        std::vector<char> host[3];
+        auto spread = [&](int k, void* dst, const void* tile, size_t bytes) -> int {
             if (!bytes) return SIM_OK;
             char* d = static_cast<char*>(dst);
-            CUDA_TRY(cudaMemcpyAsync(d, tile, bytes, cudaMemcpyHostToDevice, st));
-            for (size_t done = bytes, n; done < bytes * tiles; done += n) {
+            const size_t first = std::min(tiles, std::max<size_t>(1, (size_t(1) << 20) / bytes));
+            host[k].resize(bytes * first);
+            for (size_t t = 0; t < first; t++) memcpy(host[k].data() + t * bytes, tile, bytes);
+            CUDA_TRY(cudaMemcpyAsync(d, host[k].data(), bytes * first, cudaMemcpyHostToDevice, st));
+            for (size_t done = bytes * first, n; done < bytes * tiles; done += n) {
                 n = std::min(done, bytes * tiles - done);
                 CUDA_TRY(cudaMemcpyAsync(d + done, d, n, cudaMemcpyDeviceToDevice, st));
             }
             return SIM_OK;
         };
-        if ((rc = spread(S.bits[0], bitw.data(), bitw.size() * 4)) || (rc = spread(S.w32[0], w32.data(), w32.size() * 4)) ||
-            (rc = spread(S.w64[0], w64.data(), w64.size() * 8)))
+        if ((rc = spread(0, S.bits[0], bitw.data(), bitw.size() * 4)) ||
+            (rc = spread(1, S.w32[0], w32.data(), w32.size() * 4)) || (rc = spread(2, S.w64[0], w64.data(), w64.size() * 8)))
             return rc;
         CUDA_TRY(cudaStreamSynchronize(st));
     }
@@ -1198,6 +1257,21 @@ int step_graph(sim_batch* b, uint64_t n) {
     return SIM_OK;
 }
 
+// One instance's registers (mem < 0) or the n words of a memory: a kernel writes
+// them and the error word to pinned memory, one wait in place of a copy of the
+// error word and three strided copies with waits of their own (a step of 8
+// cycles of the 2k-op netlist and its registers: 84 -> 49 us).
+int read_back(sim_batch* b, uint32_t inst, int32_t mem, uint32_t n, uint64_t* out) {
+    if (int rc = refuse_failed(b)) return rc;
+    Stage st;
+    if (int rc = st.take()) return rc;
+    CUDA_TRY(launch_read(b->stream, b->P, b->S, uint32_t(b->cycle & 1), inst, mem, n, st.p));
+    CUDA_TRY(cudaStreamSynchronize(b->stream));
+    if (st.p[0]) return check_err(b);
+    memcpy(out, st.p + 1, size_t(n) * 8);
+    return SIM_OK;
+}
+
 sim_batch* B(void* p) { return static_cast<sim_batch*>(p); }
 
 int check_inst(sim_batch* b, uint32_t inst) {
@@ -1475,9 +1549,10 @@ int sim_peek_mems(sim_batch* b, uint32_t inst, uint32_t mem, uint64_t* out) {
     if (rc) return rc;
     const Netlist& nl = b->nl->nl;
     if (!out || mem >= nl.mem_lg.size()) return set_err(SIM_ERR_BADARG, "bad argument");
+    const size_t depth = size_t(1) << nl.mem_lg[mem];
+    if (depth < kStageBytes / 8) return read_back(b, inst, int32_t(mem), uint32_t(depth), out);
     rc = sim_sync(b);
     if (rc) return rc;
-    const size_t depth = size_t(1) << nl.mem_lg[mem];
     // instance-minor layout: word a of instance inst is at (base + a) * I + inst
     CUDA_TRY(cudaMemcpy2DAsync(out, 8, b->S.mem + b->nl->mem_word_off[mem] * b->I + inst, size_t(b->I) * 8, 8, depth,
                                cudaMemcpyDeviceToHost, b->stream));
@@ -1489,9 +1564,10 @@ int sim_peek_regs(sim_batch* b, uint32_t inst, uint64_t* out) {
     int rc = check_inst(b, inst);
     if (rc) return rc;
     if (!out) return set_err(SIM_ERR_BADARG, "null output");
+    const RegLayout& L = b->nl->layout;
+    if (L.cls.size() < kStageBytes / 8) return read_back(b, inst, -1, uint32_t(L.cls.size()), out);
     rc = sim_sync(b);
     if (rc) return rc;
-    const RegLayout& L = b->nl->layout;
     const DevState& S = b->S;
     const uint32_t par = uint32_t(b->cycle & 1);
     std::vector<uint64_t> v64(L.count[RC_W64]);
@@ -1579,21 +1655,28 @@ constexpr uint64_t kMagic = 0x314B505453525447ULL;
 
 int sim_save(sim_batch* b, void** blob, size_t* len) {
     if (!b || !blob || !len) return set_err(SIM_ERR_BADARG, "null argument");
-    int rc = sim_sync(b);
-    if (rc) return rc;
+    if (int rc = refuse_failed(b)) return rc;
     const RegLayout& L = b->nl->layout;
     const DevState& S = b->S;
-    // registers in [register][instance] order whatever the kernels' layout
-    uint32_t par = uint32_t(b->cycle & 1);
-    if (S.pack == 32) {
-        CUDA_TRY(launch_retile(b->stream, S, par, false));
-        par ^= 1;
-    }
     size_t nb = size_t(L.count[RC_BIT]) * (S.I / S.pack) * 4, n32 = size_t(L.count[RC_W32]) * S.I * 4,
            n64 = size_t(L.count[RC_W64]) * S.I * 8, nm = b->mem.n, nmd = b->mem_dig.n, nh = b->h_hold_val.size();
     size_t total = sizeof(BlobHeader) + nb + n32 + n64 + nm + nmd + nh * 9;
     char* p = static_cast<char*>(malloc(total));
     if (!p) return set_err(SIM_ERR_OOM, "host allocation failed");
+    // touch the pages while a step may still run: a copy into pages that are
+    // not mapped yet faults on the device for each (21 MB: 21 ms instead of 1.6)
+    for (size_t i = 0; i < total; i += 4096) p[i] = 0;
+    // registers in [register][instance] order whatever the kernels' layout
+    uint32_t par = uint32_t(b->cycle & 1);
+    int rc = sim_sync(b);
+    if (!rc && S.pack == 32) {
+        if (launch_retile(b->stream, S, par, false) != cudaSuccess) rc = set_err(SIM_ERR_CUDA, "checkpoint kernel failed");
+        par ^= 1;
+    }
+    if (rc) {
+        free(p);
+        return rc;
+    }
     BlobHeader h{kMagic, 1, b->nl->nl.reg_w.size(), b->nl->mem_word_off.back(), S.I, uint64_t(b->mode), b->cycle, b->nl->nl.in_w.size()};
     memcpy(p, &h, sizeof h);
     char* q = p + sizeof h;
