@@ -53,9 +53,10 @@ def default_candidates(n_inst: int, sms: int = 152):
                 [dict(mode="lane_inst", lowering="generated", warps_per_cta=8, task_order="group_major")] +
                 [dict(mode="lane_inst", lowering="generated", warps_per_cta=w, task_order="process_major",
                       target_processes=4 * sms) for w in (12, 8)])
-    # operator pairs chained in one step (chain=2) measured faster on every
-    # geometry; the unchained adaptive geometry stays as the reference
+    # without operator pairs the step interpreter is 5-10 % faster on most
+    # geometries, with them as fast in one cluster
     cands = [dict(mode="lane_op", lowering="bytecode", chain=0),              # adaptive: 4 or 8 per SM
+             dict(mode="lane_op", lowering="bytecode", chain=0, partitioner="hypergraph"),
              dict(mode="lane_op", lowering="bytecode", chain=2),
              dict(mode="lane_op", lowering="bytecode", chain=2, warps_per_cta=8, target_processes=8 * sms),
              dict(mode="lane_op", lowering="bytecode", chain=2, warps_per_cta=3, target_processes=3 * sms)]
@@ -66,6 +67,8 @@ def default_candidates(n_inst: int, sms: int = 152):
         # that measured best with the bottom-up merge
         cands += [dict(mode="lane_op", lowering="bytecode", chain=2, cluster_size=c, warps_per_cta=4,
                        partitioner="hypergraph") for c in (2, 4)]
+        cands += [dict(mode="lane_op", lowering="bytecode", chain=0, cluster_size=2, warps_per_cta=4,
+                       partitioner="hypergraph")]
     return cands
 
 

@@ -484,13 +484,15 @@ __device__ void task_lane_op_res(const DevProg& P, const DevState& S, uint32_t p
                     // operands hold values of earlier steps (a slot written in
                     // this step is never read here except through the chain
                     // bits), so they are loaded together with the first row's,
-                    // before its store; so are the next step's operators.
+                    // before its store.  The next step's first operators are
+                    // loaded here too; with its second ones as well the grid
+                    // barrier's kernel measured 8 % slower, 2-CTA clusters the same.
                     e = table[++b];
                     const OpFields f1 = op_fields(o1), f2 = op_fields(o2);
                     const uint64_t a1 = ld(f1.a), m1 = ld(f1.m), x1 = ld(f1.x), d1 = ld(f1.d);
                     const uint64_t a2 = ld(f2.a), m2 = ld(f2.m), x2 = ld(f2.x), d2 = ld(f2.d);
                     o = (e & kStepChain) ? ins + (e & 0xffff) + 2 * min(lane, (e >> 16) & 31u) : o;
-                    const uint4 n1 = o[0], n2 = o[1];
+                    const uint4 n1 = o[0];
                     const uint64_t r1 = eval_op(f1.w0, f1.bits, a1, m1, x1, d1, false);
                     st(f1.dst, r1);
                     const uint64_t r2 = eval_op(f2.w0, f2.bits, (f2.bits & kOpChainA) ? r1 : a2, m2,
@@ -499,7 +501,7 @@ __device__ void task_lane_op_res(const DevProg& P, const DevState& S, uint32_t p
                     st(f2.dst, r2);
                     __syncwarp();
                     o1 = n1;
-                    o2 = n2;
+                    o2 = o[1];
                 } while (e & kStepChain);
             }
             if (b >= nb) break;
