@@ -1678,10 +1678,13 @@ int lower(const Netlist& nl, const Partition& part, Lowered& out, std::string& e
             return (op == OP_INPUT || op == OP_REG || op == OP_CONST) ? 1 : 2;
         };
         for (auto& it : items) it.phase = phase(it);
-        std::stable_sort(items.begin(), items.end(), [](const Item& a, const Item& b) {
+        // leaves: registers first, whose loads take longest, then inputs (a
+        // hash each), then constants; so most rows of 32 are of one kind
+        auto rank = [](const Item& it) { return it.phase != 1 ? int(it.op) : it.op == OP_REG ? 0 : it.op == OP_INPUT ? 1 : 2; };
+        std::stable_sort(items.begin(), items.end(), [&](const Item& a, const Item& b) {
             if (a.phase != b.phase) return a.phase < b.phase;
             if (a.level != b.level) return a.level < b.level;
-            if (a.op != b.op) return a.op < b.op;
+            if (rank(a) != rank(b)) return rank(a) < rank(b);
             if (a.kind != b.kind) return a.kind < b.kind;
             return a.id < b.id;
         });
@@ -2278,6 +2281,10 @@ int lower_clusters(const Netlist& nl, const Partition& part, uint32_t C, uint32_
                     }
                 }
             }
+        // leaf steps: reads across clusters (L2) before those of the mirror
+        for (auto& st : steps[p])
+            if (st.flags & kStepLeaf)
+                std::stable_partition(st.ins.begin(), st.ins.end(), [](const DIns& d) { return d.op == D_LDR; });
         // without operator pairs: into the last store step while it has
         // room, then new store steps; with them: steps of 32
         const size_t width = wide_stores ? kLeafStepMax : 32;

@@ -457,12 +457,10 @@ __device__ __forceinline__ void fill_const_table(uint64_t* tab) {
 // PAIRS: the program was lowered with operator pairs, whose steps are tested
 // first (a program without them never pays that test).
 template <bool DIGEST, bool PAIRS>
-__device__ void task_lane_op_res(const DevProg& P, const DevState& S, uint32_t p, uint32_t inst, uint64_t t,
-                                 bool pending, char* sm, uint64_t* sl, const uint32_t* __restrict__ prog,
+__device__ void task_lane_op_res(const DevProg& P, const DevState& S, uint32_t p, uint32_t inst, uint64_t key,
+                                 int32_t col, uint64_t t, bool pending, char* sm, uint64_t* sl, const uint32_t* __restrict__ prog,
                                  uint32_t lane, uint32_t dummy,
                                  const uint64_t* mir_cur = nullptr, uint32_t mir_nxt = 0) {
-    const uint64_t key = S.key[inst];
-    const int32_t col = DIGEST ? S.track[inst] : -1;
     uint64_t dacc = 0;
     const uint32_t nb = prog[0];
     // (the word after the last step word is padding or a leaf's first word: no chain bit)
@@ -654,6 +652,11 @@ __global__ void __launch_bounds__(1024) k_cycles(DevProg P, DevState S, LaunchAr
         __syncthreads();
     }
     const uint64_t t_base = A.t0_dev ? *A.t0_dev + A.t0 : A.t0;
+    // the instance's stimulus key and digest column, read when it changes (not
+    // every cycle, in front of the first input's hash)
+    uint32_t g_known = ~0u;
+    uint64_t key = 0;
+    int32_t col = -1;
     uint32_t gen = 0;
     for (uint32_t c = 0; c < A.n; c++) {
         const uint64_t t = t_base + c;
@@ -663,9 +666,15 @@ __global__ void __launch_bounds__(1024) k_cycles(DevProg P, DevState S, LaunchAr
         if (resident) {
             uint32_t off = 0;
             for (uint32_t p = p_first; p < P.n_proc && g_first < A.replicas; p += p_step) {
-                for (uint32_t g = g_first; g < S.I; g += A.replicas)
-                    task_lane_op_res<DIGEST, PAIRS>(P, S, p, g, t, pending, reinterpret_cast<char*>(smem), sl, prog + off,
+                for (uint32_t g = g_first; g < S.I; g += A.replicas) {
+                    if (g != g_known) {
+                        g_known = g;
+                        key = S.key[g];
+                        col = DIGEST ? S.track[g] : -1;
+                    }
+                    task_lane_op_res<DIGEST, PAIRS>(P, S, p, g, key, col, t, pending, reinterpret_cast<char*>(smem), sl, prog + off,
                                                     lane, A.slot_words - 1);
+                }
                 off += P.c_size[p];
             }
         } else {
@@ -738,6 +747,8 @@ __global__ void __launch_bounds__(1024) k_cycles_cl(DevProg P, DevState S, Launc
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     cluster_sync_all();   // every CTA of the cluster runs; mirrors and barriers are ready
+    const uint64_t key = S.key[0];
+    const int32_t col = DIGEST ? S.track[0] : -1;
     uint32_t gen = 0;
     bool ok = true;
     for (uint32_t c = 0; c < A.n && ok; c++) {
@@ -749,7 +760,7 @@ __global__ void __launch_bounds__(1024) k_cycles_cl(DevProg P, DevState S, Launc
             const uint32_t par = uint32_t(t & 1);
             const uint64_t* mc = mirror + (uint64_t)par * A.mirror_words;
             const uint32_t mn = smem_addr(mirror + (uint64_t)(par ^ 1) * A.mirror_words);
-            task_lane_op_res<DIGEST, PAIRS>(P, S, p, 0, t, pending, reinterpret_cast<char*>(smem), sl, prog, lane,
+            task_lane_op_res<DIGEST, PAIRS>(P, S, p, 0, key, col, t, pending, reinterpret_cast<char*>(smem), sl, prog, lane,
                                             slot_words - 1, mc, mn);
         }
         const bool skip = (int32_t)blockIdx.x == A.skip_cta && c == 0;
