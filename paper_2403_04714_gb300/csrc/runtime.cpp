@@ -335,9 +335,9 @@ int sim_load_netlist(const void* text, size_t len, const sim_config* cfg, sim_ne
         // defaults measured on GB300: one process per warp of 8-warp CTAs for a
         // single instance; with lane = instance four processes per SM for the
         // bytecode and two for generated code (fewer fibers duplicated across
-        // processes: mid x 4,096 15.0-15.2M against 14.2-14.4M
-        // instance-cycles/s at four); with cluster exchange one process per
-        // warp of every resident cluster CTA
+        // processes: 200k-op netlist x 4,096 186 us a cycle against 193 at four;
+        // one, 180 us, leaves small batches too few tasks); with cluster
+        // exchange one process per warp of every resident cluster CTA
         if (!target && h->cfg.cluster_size >= 2 && h->cfg.cluster_size <= 16) {
             const uint32_t W = h->cfg.warps_per_cta ? h->cfg.warps_per_cta : 8;
             target = uint32_t(resident_clusters(h->cfg.cluster_size, W)) * h->cfg.cluster_size * W;
@@ -606,10 +606,10 @@ uint32_t resident_words(const Lowered& L, uint32_t total_warps) {
 }
 
 // The operators of a resident program address the constant table and the
-// slots of a CTA with 16-bit byte offsets.  A value takes a slot (8 bytes) and
-// at least an instruction and a half (24) on chip, so no CTA whose programs fit
-// shared memory needs more slots than that, short of one that keeps nearly
-// every value it computes until the end.
+// slots of a CTA with 16-bit byte offsets.  A value that is live takes a slot
+// (8 bytes), the instruction that made it (16) and at least a third of one that
+// takes it in (16 / 3): 64 KB of slots would need 234 KB of shared memory, more
+// than a CTA has, so every program that fits is within this.
 constexpr size_t kMaxSlotBytes = 65536;
 
 // Cluster exchange: one process per warp on the planned grid of clusters;
@@ -681,8 +681,8 @@ int plan_lane_inst(sim_batch* b, uint32_t share) {
     const Lowered& L = b->nl->low;
     const uint32_t n_proc = uint32_t(L.b_slots.size()), G = b->n_tasks / n_proc;
     const int sms = sm_count();
-    const int lo = b->cfg.warps_per_cta ? std::min(32, int(b->cfg.warps_per_cta)) : 1;
-    const int hi = b->cfg.warps_per_cta ? lo : 32;
+    int lo = b->cfg.warps_per_cta ? std::min(32, int(b->cfg.warps_per_cta)) : 1;
+    int hi = b->cfg.warps_per_cta ? lo : 32;
     const bool per_cycle = b->kernel == SIM_KERNEL_PER_CYCLE || b->kernel == SIM_KERNEL_PER_CYCLE_GRAPH;
     auto area_bytes = [&](int w, uint32_t band) {
         uint64_t words = 0;
@@ -693,29 +693,32 @@ int plan_lane_inst(sim_batch* b, uint32_t share) {
     uint64_t best = ~0ull;
     b->slot_words = 0;
     b->prog_words = 0;
-    for (int w = lo; w <= hi; w++) {
-        const int most = b->cfg.warps_per_cta ? 32 / w : 1;       // CTAs per SM
-        for (int k = std::max(1, most); k >= 1; k--) {
-            const uint32_t need = (b->n_tasks + w - 1) / w;
-            const uint32_t grid = std::max(1u, std::min(need, uint32_t(std::max(1, k * sms / int(std::max(1u, share))))));
-            const uint64_t rounds = (b->n_tasks + uint64_t(grid) * w - 1) / (uint64_t(grid) * w);
-            if (rounds >= best) continue;
-            // (launches of one cycle have a warp for every task)
-            bool banded = false;
-            size_t smem = area_bytes(w, per_cycle ? need : grid);
-            if (smem > smem_limit() && !per_cycle) banded = true, smem = area_bytes(w, uint32_t(rounds * grid));
-            if (smem > smem_limit()) continue;
-            int occ = 0;
-            CUDA_TRY(prepare_cycles_kernel(b->mode, smem));
-            CUDA_TRY(occupancy_cycles(b->mode, w * 32, smem, &occ));
-            if (uint64_t(occ) * sms < grid) continue;
-            best = rounds;
-            b->banded = banded;
-            b->warps = w;
-            b->threads = w * 32;
-            b->smem = smem;
-            b->max_grid = occ * sms;
-            b->grid = int(grid);
+    // (a configured CTA size that does not fit is halved until it does)
+    for (; best == ~0ull && lo >= 1; lo = lo / 2, hi = lo) {
+        for (int w = lo; w <= hi; w++) {
+            const int most = b->cfg.warps_per_cta ? 32 / w : 1;       // CTAs per SM
+            for (int k = std::max(1, most); k >= 1; k--) {
+                const uint32_t need = (b->n_tasks + w - 1) / w;
+                const uint32_t grid = std::max(1u, std::min(need, uint32_t(std::max(1, k * sms / int(std::max(1u, share))))));
+                const uint64_t rounds = (b->n_tasks + uint64_t(grid) * w - 1) / (uint64_t(grid) * w);
+                if (rounds >= best) continue;
+                // (launches of one cycle have a warp for every task)
+                bool banded = false;
+                size_t smem = area_bytes(w, per_cycle ? need : grid);
+                if (smem > smem_limit() && !per_cycle) banded = true, smem = area_bytes(w, uint32_t(rounds * grid));
+                if (smem > smem_limit()) continue;
+                int occ = 0;
+                CUDA_TRY(prepare_cycles_kernel(b->mode, smem));
+                CUDA_TRY(occupancy_cycles(b->mode, w * 32, smem, &occ));
+                if (uint64_t(occ) * sms < grid) continue;
+                best = rounds;
+                b->banded = banded;
+                b->warps = w;
+                b->threads = w * 32;
+                b->smem = smem;
+                b->max_grid = occ * sms;
+                b->grid = int(grid);
+            }
         }
     }
     if (best == ~0ull) return set_err(SIM_ERR_CAPACITY, "the processes' value slots do not fit a CTA's shared memory");
@@ -782,14 +785,14 @@ int plan_launch(sim_batch* b) {
     int warps = b->cfg.warps_per_cta ? int(b->cfg.warps_per_cta) : 8;
     if (!b->cfg.warps_per_cta && b->mode == SIM_MODE_LANE_OP)   // one process per warp, one CTA per SM
         warps = int(std::min<uint64_t>(16, std::max<uint64_t>(1, (uint64_t(n_proc) * b->I + sms - 1) / sms)));
-    if (b->mode == SIM_MODE_LANE_INST && b->proc_major && !b->wave_groups) return plan_lane_inst(b, 1);
+    if (b->mode == SIM_MODE_LANE_INST && b->proc_major && !b->wave_groups && n_proc) return plan_lane_inst(b, 1);
     while (warps > 1 && size_t(warps) * slot_bytes > smem_cap) warps /= 2;
     b->warps = warps;
     b->threads = warps * 32;
     b->prog_words = 0;
     int occ = 0;
     b->replicas = 1;
-    if (b->mode == SIM_MODE_LANE_OP && b->I > 1) {
+    if (b->mode == SIM_MODE_LANE_OP && b->I > 1 && n_proc) {
         int rc = plan_replicas(b, slot_bytes);
         if (rc || b->replicas > 1) return rc;
     }

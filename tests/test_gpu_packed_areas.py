@@ -40,3 +40,13 @@ def test_bands_with_memories():
         ref = oracle.Sim(net, seed=6, inst=i)
         ref.run(30)
         assert got[i] == ref.digest(), i
+
+
+def test_configured_warps_that_do_not_fit():
+    # 32 warps' slots of the 200k-op netlist exceed an SM: fewer run
+    b = sim.Batch(sim.Netlist(open(netgen.cached_netlist("mid")).read(), mode="lane_inst", warps_per_cta=32), 33, seed=1)
+    assert 1 <= b.launch_info()["warps_per_cta"] < 32
+    b.step(5)
+    ref = oracle.Sim(oracle.Net(text=open(netgen.cached_netlist("mid")).read()), seed=1, inst=32)
+    ref.run(5)
+    assert b.state_digests()[32] == ref.digest()
