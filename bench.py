@@ -35,8 +35,8 @@ STATE_BYTES_MID = 6126 / 8 + 7955 * 4 + 5927 * 8
 # the headline kernel (ncu, 1 pass): the one-time program and table load; the
 # per-cycle exchange stays in L2 (capture: ncu --metrics dram__bytes_read.sum,
 # dram__bytes_write.sum -k regex:k_cycles -s 1 -c 1 on `bench.py --no-rows
-# --steps 2 --warmup 1`, operator pairs in 2-CTA clusters, hypergraph partition)
-HEADLINE_TRAFFIC = 5.218e6 + 0.104e6
+# --steps 2 --warmup 1`, 2-CTA clusters, hypergraph partition)
+HEADLINE_TRAFFIC = 5.068e6 + 0.092e6
 HBM_PEAK_GBS = 6790.0       # overwritten from MEASURED_PEAKS.json when present
 WORKLOAD = ("mid netlist: 200k ops, 20k registers (30% 1b / 40% 32b / 30% 64b), depth 60, "
             "fan-out power law (alpha 2, max 512), two 512x64b synchronous RAMs; 1 instance, "

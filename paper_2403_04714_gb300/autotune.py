@@ -43,11 +43,10 @@ def _key(text: bytes, n_inst: int, device: str) -> str:
 
 def default_candidates(n_inst: int, sms: int = 152):
     if n_inst >= 32:
-        # each warp's staging area of shared memory bounds the warps per SM:
-        # smaller CTAs let more of them share an SM.  The default partition
-        # has two processes per SM (fewer fibers duplicated across processes
-        # than with four: mid 210k instead of 220k generated instructions per
-        # instance-cycle, measured 4-7 % faster); four stay candidates
+        # CTAs of 8 and more warps measure alike, of 4 and 6 behind them when
+        # their rounds do not fill the GPU.  The default partition has two
+        # processes per SM (fewer fibers duplicated across processes than with
+        # four); four stay candidates
         return ([dict(mode="lane_inst", lowering="generated", warps_per_cta=w, task_order="process_major")
                  for w in (12, 8, 6, 4)] +
                 [dict(mode="lane_inst", lowering="generated", warps_per_cta=8, task_order="group_major")] +

@@ -16,7 +16,7 @@ typedef long long int64_t;
 
 namespace rtl {
 
-// Register storage classes (instance-minor planes on the device).
+// Register storage classes (a plane each on the device).
 enum RegClass : uint8_t { RC_BIT = 0, RC_W32 = 1, RC_W64 = 2 };
 
 // ------------------------------------------------------------------------

@@ -1493,7 +1493,10 @@ int append_program(const std::vector<CStep>& steps, std::vector<uint32_t>& words
 // store and an evaluation) to the whole step.  A variant
 // that kept only the pairs' second operators (no D_NOP, lanes with a pair
 // first) made smaller programs but measured 4 % slower on the same GPU
-// (79.3k against 82.6k cycles/s), so the rows stay full.
+// (79.3k against 82.6k cycles/s), so the rows stay full.  (Those figures are of
+// an evaluator that cost two thirds more a row.  With operators as one formula
+// a step without pairs is cheap enough that pairs are 5-10 % slower, 8.8
+// against 8.4 us a cycle, except in a grid of one cluster, 3.17 against 3.20.)
 template <class MakeIns, class Operands>
 int chained_program(const Netlist& nl, const std::vector<Item>& items, const std::vector<int32_t>& local, size_t n_local,
                     MakeIns& make_ins, Operands& operands, Lowered& out, size_t p, uint32_t K, std::string& err) {

@@ -16,7 +16,7 @@
 //   LANE_OP   warp = (process, instance); lanes run up to 32 independent
 //             nodes of one schedule step, __syncwarp between steps.
 //   LANE_INST warp = (process, 32 instances); lane = instance, uniform
-//             control flow, instance-minor state (coalesced 128/256 B rows),
+//             control flow, state in tiles of 32 instances (coalesced 128/256 B rows),
 //             1-bit registers packed 32 instances per word with __ballot_sync.
 #include <cuda_runtime.h>
 
