@@ -54,9 +54,10 @@ constexpr uint32_t kStepLeaf = 1u << 30;
 // rows also read as sequential steps).
 constexpr uint32_t kStepChain = 1u << 29;
 // A store step (also kStepGeneric) holds only register stores (D_STR) and
-// mirror stores (D_STX), up to kLeafStepMax of them, four per lane.  Only
-// programs without operator pairs have them (measured: with pairs the store
-// step's code slows the pair loop more than the steps it saves).
+// mirror stores (D_STX), up to kLeafStepMax of them, four per lane.  Compact
+// programs have them without operator pairs; the device form merges
+// neighbouring store steps of every program into them (encode_programs: pairs
+// in 2-CTA clusters 8.41 -> 7.75 us a cycle, in one cluster 3.06 -> 2.84).
 constexpr uint32_t kStepStore = 1u << 28;
 constexpr uint32_t kStepRowsShift = 24;
 constexpr uint32_t kStepRowsMask = 0xfu;

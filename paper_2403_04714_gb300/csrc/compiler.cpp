@@ -1495,8 +1495,9 @@ int append_program(const std::vector<CStep>& steps, std::vector<uint32_t>& words
 // first) made smaller programs but measured 4 % slower on the same GPU
 // (79.3k against 82.6k cycles/s), so the rows stay full.  (Those figures are of
 // an evaluator that cost two thirds more a row.  With operators as one formula
-// a step without pairs is cheap enough that pairs are 5-10 % slower, 8.8
-// against 8.4 us a cycle, except in a grid of one cluster, 3.17 against 3.20.)
+// a step without pairs is cheap enough that pairs are as fast with cluster
+// exchange, 7.7 us a cycle either way, and slower on the grid barrier with two
+// warps per scheduler, 11.7 against 10.4 on the 499k-op mesh.)
 template <class MakeIns, class Operands>
 int chained_program(const Netlist& nl, const std::vector<Item>& items, const std::vector<int32_t>& local, size_t n_local,
                     MakeIns& make_ins, Operands& operands, Lowered& out, size_t p, uint32_t K, std::string& err) {
@@ -2030,16 +2031,30 @@ void encode_programs(Lowered& low) {
         const DIns* ins = reinterpret_cast<const DIns*>(w + tw);
         uint32_t* out = low.e_words.data() + low.c_off[p] + tw;
         low.e_tab[p] = tw / 4;
+        uint32_t* table = low.e_words.data() + low.c_off[p] + 1;
+        uint32_t ne = 0;                        // steps of the device form
         for (uint32_t b = 0; b < nb; b++) {
             const uint32_t e = w[1 + b], first = e & 0xffff, cnt = (e >> 16) & kStepCountMask;
             const bool pair = e & kStepChain;
-            if (!pair && (e & kStepGeneric)) continue;
+            if (!pair && (e & kStepGeneric)) {
+                // register and mirror stores of neighbouring steps form wide store steps
+                bool stores = !(e & kStepLeaf) && cnt > 0;
+                for (uint32_t i = 0; i < cnt && stores; i++) stores = ins[first + i].op == D_STR || ins[first + i].op == D_STX;
+                const uint32_t last = ne ? table[ne - 1] : 0, have = (last >> 16) & kStepCountMask;
+                if (stores && (last & kStepStore) && have + cnt <= kLeafStepMax)
+                    table[ne - 1] = (last & ~(kStepCountMask << 16)) | (have + cnt) << 16;
+                else
+                    table[ne++] = e | (stores ? kStepStore : 0u);
+                continue;
+            }
             // a lane's two operators side by side; step words hold the last lane
             const uint32_t n = pair ? cnt / 2 : cnt;
             for (uint32_t i = 0; i < cnt; i++)
                 encode_op(ins[first + i], i >= n, out + size_t(first + (pair ? i % n * 2 + i / n : i)) * 4);
-            low.e_words[low.c_off[p] + 1 + b] = (e & ~(kStepCountMask << 16)) | (n - 1) << 16;
+            table[ne++] = (e & ~(kStepCountMask << 16)) | (n - 1) << 16;
         }
+        for (uint32_t b = ne; b < nb; b++) table[b] = 0;
+        low.e_words[low.c_off[p]] = ne | (tw / 4) << 16;
     }
 }
 

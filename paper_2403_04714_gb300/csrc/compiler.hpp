@@ -122,7 +122,9 @@ int lower(const Netlist& nl, const Partition& part, Lowered& out, std::string& e
 // The device form of the compact programs: the operators of operator and chain
 // steps as instances of one formula (kOpMark), a chain step's pairs side by
 // side, and those steps' words with the number of their last lane in place of
-// the instruction count; everything else as it is.
+// the instruction count; neighbouring steps of stores merged into wide store
+// steps; everything else as it is.  Word 0: steps | 16-byte units before the
+// instructions << 16.
 void encode_programs(Lowered& low);
 
 // Cluster exchange.  Processes are placed on a grid of thread-block

@@ -462,10 +462,10 @@ __device__ void task_lane_op_res(const DevProg& P, const DevState& S, uint32_t p
                                  uint32_t lane, uint32_t dummy,
                                  const uint64_t* mir_cur = nullptr, uint32_t mir_nxt = 0) {
     uint64_t dacc = 0;
-    const uint32_t nb = prog[0];
+    const uint32_t nb = prog[0] & 0xffffu;
     // (the word after the last step word is padding or a leaf's first word: no chain bit)
     const uint32_t* table = prog + 1;
-    const uint4* ins = reinterpret_cast<const uint4*>(prog + ((nb + 4) & ~3u));
+    const uint4* ins = reinterpret_cast<const uint4*>(prog) + (prog[0] >> 16);
     const auto ld = [&](uint32_t off) { return *reinterpret_cast<const uint64_t*>(sm + off); };
     const auto st = [&](uint32_t off, uint64_t v) { *reinterpret_cast<uint64_t*>(sm + off) = v; };
     uint32_t e = table[0];
@@ -526,9 +526,9 @@ __device__ void task_lane_op_res(const DevProg& P, const DevState& S, uint32_t p
         if (PAIRS && !(e & kStepGeneric)) {
             const OpFields f = op_fields(ins[first + min(lane, cnt)]);      // operator step
             st(f.dst, eval_op(f.w0, f.bits, ld(f.a), ld(f.m), ld(f.x), ld(f.d), false));
-        } else if (!PAIRS && (e & kStepStore)) {
-            // programs without pairs: up to four register or mirror stores per
-            // lane, every slot value loaded before the first store
+        } else if (e & kStepStore) {
+            // up to four register or mirror stores per lane, every slot value
+            // loaded before the first store
             uint4 raw[4];
             uint64_t v[4];
 #pragma unroll
