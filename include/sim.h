@@ -134,8 +134,8 @@ typedef struct sim_config {
                                  * alternative strategy of Sec. 7) */
     uint32_t chain;             /* LANE_OP shared-memory programs: 2 = a lane may run a dependent pair of operators
                                  * in one step (the first result passed on in a register), 0/1 = one dependence
-                                 * level per step (the default).  Pairs are as fast in a grid of one cluster and
-                                 * 5-10 % slower elsewhere (measured on GB300). */
+                                 * level per step (the default).  Either is up to 5 % faster, by design
+                                 * and geometry (measured on GB300; the autotuner tries both). */
     uint32_t reserved[1];
 } sim_config;
 

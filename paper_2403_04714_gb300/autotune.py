@@ -52,8 +52,8 @@ def default_candidates(n_inst: int, sms: int = 152):
                 [dict(mode="lane_inst", lowering="generated", warps_per_cta=8, task_order="group_major")] +
                 [dict(mode="lane_inst", lowering="generated", warps_per_cta=w, task_order="process_major",
                       target_processes=4 * sms) for w in (12, 8)])
-    # without operator pairs the step interpreter is 5-10 % faster on most
-    # geometries, with them as fast in one cluster
+    # with and without operator pairs the step interpreter is within 5 %,
+    # either way round by design and geometry
     cands = [dict(mode="lane_op", lowering="bytecode", chain=0),              # adaptive: 4 or 8 per SM
              dict(mode="lane_op", lowering="bytecode", chain=0, partitioner="hypergraph"),
              dict(mode="lane_op", lowering="bytecode", chain=2),

@@ -1495,9 +1495,8 @@ int append_program(const std::vector<CStep>& steps, std::vector<uint32_t>& words
 // first) made smaller programs but measured 4 % slower on the same GPU
 // (79.3k against 82.6k cycles/s), so the rows stay full.  (Those figures are of
 // an evaluator that cost two thirds more a row.  With operators as one formula
-// a step without pairs is cheap enough that pairs are as fast with cluster
-// exchange, 7.7 us a cycle either way, and slower on the grid barrier with two
-// warps per scheduler, 11.7 against 10.4 on the 499k-op mesh.)
+// the two are within 5 %: 200k-op netlist in 2-CTA clusters 7.85 us a cycle with
+// pairs, 7.94 without; 499k-op mesh, two warps per scheduler, 10.9 against 10.4.)
 template <class MakeIns, class Operands>
 int chained_program(const Netlist& nl, const std::vector<Item>& items, const std::vector<int32_t>& local, size_t n_local,
                     MakeIns& make_ins, Operands& operands, Lowered& out, size_t p, uint32_t K, std::string& err) {
