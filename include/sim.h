@@ -322,6 +322,12 @@ int sim_phase_times(sim_batch *b, uint32_t n, double *out);
  * returns SIM_ERR_TIMEOUT.  No fault, trap or unbounded wait is involved. */
 int sim_debug_skip_arrival(sim_batch *b, uint32_t timeout_ms);
 
+/* Testing hook: the launch plan that the lane = instance bytecode of `groups`
+ * x 32 instances gets on 1 / share of a GB300 (152 SMs), worked out without a
+ * GPU: out = CTAs, warps per CTA, rounds of tasks, banded (0/1), shared memory
+ * of a CTA in bytes, CTAs that fit on the GPU.  Errors: BADARG, CAPACITY. */
+int sim_debug_lane_plan(const sim_netlist *nl, uint32_t groups, uint32_t share, int32_t per_cycle, uint64_t *out);
+
 /* ---- serving: continuous batching of simulation jobs ---------------------
  * The paper motivates simulation throughput by many regression runs of one
  * design (Sec. 1 and the nightly-regression cost model of Sec. 6, Cost

@@ -16,6 +16,7 @@
 #include "codegen.hpp"
 #include "compiler.hpp"
 #include "device.hpp"
+#include "lane_plan.hpp"
 
 namespace rtl {
 cudaError_t prepare_cycles_kernel(int mode, size_t smem);
@@ -674,54 +675,36 @@ int plan_launch_cluster(sim_batch* b) {
     return SIM_OK;
 }
 
-// Lane = instance bytecode, areas packed by process (lane_inst_packed): the
-// CTA size and grid on 1 / share of the GPU with the fewest rounds of tasks,
-// then the fewest warps.  CTA 0 has the largest areas.
+// Lane = instance bytecode, areas packed by process: the plan for b->n_tasks on
+// 1 / share of the GPU.
 int plan_lane_inst(sim_batch* b, uint32_t share) {
     const Lowered& L = b->nl->low;
-    const uint32_t n_proc = uint32_t(L.b_slots.size()), G = b->n_tasks / n_proc;
-    const int sms = sm_count();
-    int lo = b->cfg.warps_per_cta ? std::min(32, int(b->cfg.warps_per_cta)) : 1;
-    int hi = b->cfg.warps_per_cta ? lo : 32;
-    const bool per_cycle = b->kernel == SIM_KERNEL_PER_CYCLE || b->kernel == SIM_KERNEL_PER_CYCLE_GRAPH;
-    auto area_bytes = [&](int w, uint32_t band) {
-        uint64_t words = 0;
-        for (int i = 0; i < w && uint64_t(i) * band < b->n_tasks; i++)
-            words += L.b_slots[b->nl->b_order[size_t(i) * band / G]] * 32ull + kBlockWords;
-        return size_t(words) * 8;
-    };
-    uint64_t best = ~0ull;
+    LanePlanInput in;
+    in.n_proc = uint32_t(L.b_slots.size());
+    in.groups = b->n_tasks / in.n_proc;
+    in.sms = sm_count();
+    in.share = share;
+    in.smem_limit = smem_limit();
+    in.warps = b->cfg.warps_per_cta;
+    in.per_cycle = b->kernel == SIM_KERNEL_PER_CYCLE || b->kernel == SIM_KERNEL_PER_CYCLE_GRAPH;
+    LanePlan plan;
+    const int rc = plan_lane(in, [&](size_t i) { return L.b_slots[b->nl->b_order[i]]; },
+                             [&](int threads, size_t smem, int* ctas) -> int {
+                                 CUDA_TRY(prepare_cycles_kernel(b->mode, smem));
+                                 CUDA_TRY(occupancy_cycles(b->mode, threads, smem, ctas));
+                                 return SIM_OK;
+                             },
+                             plan);
+    if (rc) return rc;
+    if (!plan.warps) return set_err(SIM_ERR_CAPACITY, "the processes' value slots do not fit a CTA's shared memory");
     b->slot_words = 0;
     b->prog_words = 0;
-    // (a configured CTA size that does not fit is halved until it does)
-    for (; best == ~0ull && lo >= 1; lo = lo / 2, hi = lo) {
-        for (int w = lo; w <= hi; w++) {
-            const int most = b->cfg.warps_per_cta ? 32 / w : 1;       // CTAs per SM
-            for (int k = std::max(1, most); k >= 1; k--) {
-                const uint32_t need = (b->n_tasks + w - 1) / w;
-                const uint32_t grid = std::max(1u, std::min(need, uint32_t(std::max(1, k * sms / int(std::max(1u, share))))));
-                const uint64_t rounds = (b->n_tasks + uint64_t(grid) * w - 1) / (uint64_t(grid) * w);
-                if (rounds >= best) continue;
-                // (launches of one cycle have a warp for every task)
-                bool banded = false;
-                size_t smem = area_bytes(w, per_cycle ? need : grid);
-                if (smem > smem_limit() && !per_cycle) banded = true, smem = area_bytes(w, uint32_t(rounds * grid));
-                if (smem > smem_limit()) continue;
-                int occ = 0;
-                CUDA_TRY(prepare_cycles_kernel(b->mode, smem));
-                CUDA_TRY(occupancy_cycles(b->mode, w * 32, smem, &occ));
-                if (uint64_t(occ) * sms < grid) continue;
-                best = rounds;
-                b->banded = banded;
-                b->warps = w;
-                b->threads = w * 32;
-                b->smem = smem;
-                b->max_grid = occ * sms;
-                b->grid = int(grid);
-            }
-        }
-    }
-    if (best == ~0ull) return set_err(SIM_ERR_CAPACITY, "the processes' value slots do not fit a CTA's shared memory");
+    b->banded = plan.banded;
+    b->warps = plan.warps;
+    b->threads = plan.warps * 32;
+    b->smem = plan.smem;
+    b->max_grid = plan.max_grid;
+    b->grid = plan.grid;
     return SIM_OK;
 }
 
@@ -1785,6 +1768,29 @@ int sim_debug_skip_arrival(sim_batch* b, uint32_t timeout_ms) {
     if (b->grid < 2) return set_err(SIM_ERR_STATE, "needs at least two CTAs");
     b->skip_cta = 0;
     b->skip_timeout_ns = uint64_t(timeout_ms) * 1000000ULL;
+    return SIM_OK;
+}
+
+int sim_debug_lane_plan(const sim_netlist* nl, uint32_t groups, uint32_t share, int32_t per_cycle, uint64_t* out) {
+    if (!nl || !groups || !out || nl->low.b_slots.empty()) return set_err(SIM_ERR_BADARG, "bad argument");
+    LanePlanInput in;
+    in.n_proc = uint32_t(nl->low.b_slots.size());
+    in.groups = groups;
+    in.sms = 152;
+    in.share = share;
+    in.smem_limit = 227 * 1024 - 32;
+    in.warps = nl->cfg.warps_per_cta;
+    in.per_cycle = per_cycle != 0;
+    LanePlan plan;
+    plan_lane(in, [&](size_t i) { return nl->low.b_slots[nl->b_order[i]]; },
+              [](int threads, size_t smem, int* ctas) {     // 64 registers a thread, 1 KB kept by the system per CTA
+                  *ctas = int(std::min<size_t>(65536 / 64 / threads, 228 * 1024 / (smem + 1024 + 32)));
+                  return 0;
+              },
+              plan);
+    if (!plan.warps) return set_err(SIM_ERR_CAPACITY, "the processes' value slots do not fit a CTA's shared memory");
+    const uint64_t v[6] = {uint64_t(plan.grid), uint64_t(plan.warps), plan.rounds, plan.banded, plan.smem, uint64_t(plan.max_grid)};
+    std::copy(v, v + 6, out);
     return SIM_OK;
 }
 

@@ -94,6 +94,7 @@ EXPORTS = {
     "sim_free_blob": (None, [C.c_void_p]),
     "sim_launch_info": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
     "sim_debug_skip_arrival": (C.c_int, [C.c_void_p, C.c_uint32]),
+    "sim_debug_lane_plan": (C.c_int, [C.c_void_p, C.c_uint32, C.c_uint32, C.c_int32, C.c_void_p]),
     "sim_last_error": (C.c_char_p, []),
     "sim_netlist_table": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p]),
     "sim_state_digests_noalloc": (C.c_int, [C.c_void_p, C.c_void_p]),
@@ -219,6 +220,12 @@ class Netlist:
         raw = np.zeros(n.value, dtype=np.uint8)
         _check(lib().sim_netlist_table(self._h, which, raw.ctypes.data, C.byref(n)))
         return raw.view(DINS if dt is None else dt)
+
+    def debug_lane_plan(self, groups: int, share: int = 1, per_cycle: bool = False) -> dict:
+        """sim_debug_lane_plan: launch plan of the lane = instance bytecode on a GB300 (no GPU needed)."""
+        out = np.zeros(6, dtype=np.uint64)
+        _check(lib().sim_debug_lane_plan(self._h, groups, share, per_cycle, out.ctypes.data))
+        return dict(zip(("ctas", "warps_per_cta", "rounds", "banded", "smem", "max_ctas"), map(int, out)))
 
     def info(self) -> dict:
         out = sim_netlist_info()

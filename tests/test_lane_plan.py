@@ -1,0 +1,32 @@
+"""Launch plans of the lane = instance bytecode (CPU only): a pool on 1 / share
+of the GPU takes at most that share of the CTAs that fit, also with a configured
+CTA size whose value slots leave room for fewer CTAs per SM than its warps
+would."""
+import pytest
+
+from paper_2403_04714_gb300 import netgen, sim
+
+
+@pytest.fixture(scope="module")
+def mid_text():
+    return open(netgen.cached_netlist("mid")).read()
+
+
+@pytest.mark.parametrize("warps", [0, 4, 8, 16, 22, 32])
+def test_a_pool_keeps_to_its_share(mid_text, warps):
+    nl = sim.Netlist(mid_text, mode="lane_inst", warps_per_cta=warps)
+    tasks = nl.info()["n_processes"]
+    for groups in (1, 3, 32, 128):
+        for share in (1, 2, 3, 5, 200):
+            for per_cycle in (False, True):
+                p = nl.debug_lane_plan(groups, share, per_cycle)
+                assert 1 <= p["ctas"] <= max(1, p["max_ctas"] // share), (groups, share, p)
+                assert p["rounds"] * p["ctas"] * p["warps_per_cta"] >= tasks * groups
+                assert p["smem"] <= 227 * 1024 - 32
+                assert not (per_cycle and p["banded"])
+
+
+def test_a_configured_cta_size_is_kept_where_it_fits(mid_text):
+    for warps in (1, 4, 8):
+        nl = sim.Netlist(mid_text, mode="lane_inst", warps_per_cta=warps)
+        assert nl.debug_lane_plan(128)["warps_per_cta"] == warps
