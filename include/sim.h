@@ -322,6 +322,11 @@ int sim_phase_times(sim_batch *b, uint32_t n, double *out);
  * returns SIM_ERR_TIMEOUT.  No fault, trap or unbounded wait is involved. */
 int sim_debug_skip_arrival(sim_batch *b, uint32_t timeout_ms);
 
+/* Testing hook: how often the library has done something since it was loaded.
+ * SIM_COUNT_PLANS: searches for the launch plan of a lane = instance batch. */
+enum { SIM_COUNT_PLANS = 0, SIM_COUNT_KINDS };
+uint64_t sim_debug_count(int32_t what);
+
 /* Testing hook: the launch plan that the lane = instance bytecode of `groups`
  * x 32 instances gets on 1 / share of a GB300 (152 SMs), worked out without a
  * GPU: out = CTAs, warps per CTA, rounds of tasks, banded (0/1), shared memory

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -45,6 +46,7 @@ namespace {
 
 thread_local std::string g_err;
 constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ULL;
+std::atomic<uint64_t> g_counts[SIM_COUNT_KINDS];     // sim_debug_count
 
 int set_err(int code, const std::string& msg) {
     g_err = msg;
@@ -247,6 +249,7 @@ struct sim_batch {
     uint32_t slot_words = 0, prog_words = 0, n_tasks = 0;
     uint32_t banded = 0;                    // packed LANE_INST areas (see LaunchArgs)
     uint32_t replicas = 1;                  // warps per process (see LaunchArgs)
+    uint32_t plan_share = 1;                // share of the GPU that the plan is for (0: no plan)
     uint32_t proc_major = 0;                // task order (see LaunchArgs)
     uint32_t wave_groups = 0;
     uint32_t cta_major = 0;
@@ -549,6 +552,7 @@ int ensure_loaded(sim_netlist* h, int mode, bool digest) {
 // instances each: 24.3 us a cycle with 8 warps per CTA, 14.9 with 2; 64
 // instances: 18.2 with 8, 15.1 with 4); from 8 per SM on, 8 or more measured best.
 int plan_grid_gen(sim_batch* b, uint32_t share) {
+    g_counts[SIM_COUNT_PLANS]++;
     const int sms = sm_count();
     const int spread = int(std::min<uint32_t>(8, std::max<uint32_t>(2, (b->n_tasks + sms - 1) / sms)));
     b->warps = std::min(32, b->cfg.warps_per_cta ? int(b->cfg.warps_per_cta) : spread);
@@ -678,6 +682,7 @@ int plan_launch_cluster(sim_batch* b) {
 // Lane = instance bytecode, areas packed by process: the plan for b->n_tasks on
 // 1 / share of the GPU.
 int plan_lane_inst(sim_batch* b, uint32_t share) {
+    g_counts[SIM_COUNT_PLANS]++;
     const Lowered& L = b->nl->low;
     LanePlanInput in;
     in.n_proc = uint32_t(L.b_slots.size());
@@ -1771,6 +1776,8 @@ int sim_debug_skip_arrival(sim_batch* b, uint32_t timeout_ms) {
     return SIM_OK;
 }
 
+uint64_t sim_debug_count(int32_t what) { return what >= 0 && what < SIM_COUNT_KINDS ? g_counts[what].load() : 0; }
+
 int sim_debug_lane_plan(const sim_netlist* nl, uint32_t groups, uint32_t share, int32_t per_cycle, uint64_t* out) {
     if (!nl || !groups || !out || nl->low.b_slots.empty()) return set_err(SIM_ERR_BADARG, "bad argument");
     LanePlanInput in;
@@ -1909,13 +1916,22 @@ int pool_step(sim_batch* b, uint64_t n, uint64_t* kernels) {
 int pool_set_active(sim_batch* b, uint32_t n_groups, uint32_t share) {
     if (!b || !b->pool || b->mode != SIM_MODE_LANE_INST || n_groups == 0 || uint64_t(n_groups) * 32 > b->I)
         return set_err(SIM_ERR_BADARG, "bad active group count");
-    b->n_tasks = uint32_t(b->nl->part.procs.size()) * n_groups;
+    share = std::max(1u, share);
+    const uint32_t n_tasks = uint32_t(b->nl->part.procs.size()) * n_groups;
+    // a server's steps mostly follow one another with the same groups and
+    // share: the plan stands (the search has an occupancy query per CTA size)
+    if (n_tasks == b->n_tasks && share == b->plan_share) return SIM_OK;
+    b->n_tasks = n_tasks;
+    b->plan_share = 0;
     // a persistent step holds only the CTAs its tasks need, and at most its
     // share of the GPU, leaving the other SMs to the pools of other netlists
-    if (b->generated) return plan_grid_gen(b, share);
-    if (b->slot_words == 0) return plan_lane_inst(b, share);
-    const int cap = std::max(1, b->max_grid / int(std::max(1u, share)));
-    b->grid = std::max(1, std::min(int((b->n_tasks + b->warps - 1) / b->warps), cap));
+    if (b->generated || b->slot_words == 0) {
+        if (int rc = b->generated ? plan_grid_gen(b, share) : plan_lane_inst(b, share)) return rc;
+    } else {
+        const int cap = std::max(1, b->max_grid / int(share));
+        b->grid = std::max(1, std::min(int((b->n_tasks + b->warps - 1) / b->warps), cap));
+    }
+    b->plan_share = share;
     return SIM_OK;
 }
 

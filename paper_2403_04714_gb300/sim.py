@@ -94,6 +94,7 @@ EXPORTS = {
     "sim_free_blob": (None, [C.c_void_p]),
     "sim_launch_info": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
     "sim_debug_skip_arrival": (C.c_int, [C.c_void_p, C.c_uint32]),
+    "sim_debug_count": (C.c_uint64, [C.c_int32]),
     "sim_debug_lane_plan": (C.c_int, [C.c_void_p, C.c_uint32, C.c_uint32, C.c_int32, C.c_void_p]),
     "sim_last_error": (C.c_char_p, []),
     "sim_netlist_table": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p]),
@@ -181,6 +182,14 @@ def default_config(**kw) -> sim_config:
             v = PARTITIONERS[v]
         setattr(cfg, k, v)
     return cfg
+
+
+SIM_COUNT_PLANS = 0
+
+
+def debug_count(what: int) -> int:
+    """sim_debug_count: how often the library has done something since it was loaded."""
+    return lib().sim_debug_count(what)
 
 
 def measure_int_peak(iters: int = 4096) -> float:
