@@ -323,8 +323,9 @@ int sim_phase_times(sim_batch *b, uint32_t n, double *out);
 int sim_debug_skip_arrival(sim_batch *b, uint32_t timeout_ms);
 
 /* Testing hook: how often the library has done something since it was loaded.
- * SIM_COUNT_PLANS: searches for the launch plan of a lane = instance batch. */
-enum { SIM_COUNT_PLANS = 0, SIM_COUNT_KINDS };
+ * SIM_COUNT_PLANS: searches for the launch plan of a lane = instance batch;
+ * SIM_COUNT_PINNED: allocations of pinned memory for read-backs. */
+enum { SIM_COUNT_PLANS = 0, SIM_COUNT_PINNED, SIM_COUNT_KINDS };
 uint64_t sim_debug_count(int32_t what);
 
 /* Testing hook: the launch plan that the lane = instance bytecode of `groups`

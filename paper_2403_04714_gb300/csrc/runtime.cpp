@@ -143,46 +143,47 @@ int upload(DBuf& b, const std::vector<T>& v, cudaStream_t st) {
 
 }  // namespace
 
-// Pinned host buffers of read-backs, shared by the batches of the process: a
-// call takes one for its duration (any thread, any stream), at most
-// kStageBuffers are kept, and the last batch's end frees them.
+// Pinned host buffers of read-backs, shared by a netlist's batches: a call takes
+// one for its duration (any thread, any stream), at most kStageBuffers are kept,
+// and the end of the netlist frees them.  They belong to the netlist rather than
+// to its batches because a program that creates, steps, reads and closes one
+// batch after another would pin and unpin the memory for each.
 namespace {
-constexpr size_t kStageBytes = 1 << 20;
+constexpr size_t kStageBytes = 1 << 20;     // longer read-backs are copied without one
 constexpr size_t kStageBuffers = 4;
-std::mutex g_stage_mu;
-std::vector<void*> g_stage_free;
-size_t g_stage_users = 0;
 
-void stage_retain() {
-    std::lock_guard<std::mutex> g(g_stage_mu);
-    g_stage_users++;
-}
-void stage_release() {
-    std::lock_guard<std::mutex> g(g_stage_mu);
-    if (--g_stage_users) return;
-    for (void* p : g_stage_free) cudaFreeHost(p);
-    g_stage_free.clear();
-}
+struct StagePool {
+    size_t bytes = 8;                       // the error word and the longest read-back
+    std::mutex mu;
+    std::vector<void*> kept;
+    ~StagePool() {
+        for (void* p : kept) cudaFreeHost(p);
+    }
+};
+
 struct Stage {
+    StagePool& pool;
     uint64_t* p = nullptr;
+    explicit Stage(StagePool& s) : pool(s) {}
     int take() {
         {
-            std::lock_guard<std::mutex> g(g_stage_mu);
-            if (!g_stage_free.empty()) {
-                p = static_cast<uint64_t*>(g_stage_free.back());
-                g_stage_free.pop_back();
+            std::lock_guard<std::mutex> g(pool.mu);
+            if (!pool.kept.empty()) {
+                p = static_cast<uint64_t*>(pool.kept.back());
+                pool.kept.pop_back();
                 return SIM_OK;
             }
         }
         void* v = nullptr;
-        CUDA_TRY(cudaHostAlloc(&v, kStageBytes, cudaHostAllocPortable | cudaHostAllocMapped));
+        CUDA_TRY(cudaHostAlloc(&v, pool.bytes, cudaHostAllocPortable | cudaHostAllocMapped));
+        g_counts[SIM_COUNT_PINNED]++;
         p = static_cast<uint64_t*>(v);
         return SIM_OK;
     }
     ~Stage() {
         if (!p) return;
-        std::lock_guard<std::mutex> g(g_stage_mu);
-        if (g_stage_free.size() < kStageBuffers) g_stage_free.push_back(p);
+        std::lock_guard<std::mutex> g(pool.mu);
+        if (pool.kept.size() < kStageBuffers) pool.kept.push_back(p);
         else cudaFreeHost(p);
     }
 };
@@ -211,6 +212,7 @@ struct sim_netlist {
     std::vector<uint32_t> b_order;        // processes by descending LANE_INST slots
     std::vector<uint32_t> g_order;        // processes by descending cost
     std::vector<uint64_t> mem_word_off;   // per-instance word offset of each memory (+ total)
+    StagePool stage;                      // pinned read-back buffers of the batches
 };
 
 namespace rtl { struct PoolExtra; void pool_extra_free(PoolExtra*); }
@@ -273,9 +275,7 @@ struct sim_batch {
     DevState graph_state{};               // state descriptor captured in the graph
     bool own_stream = false;
     int device = 0;                        // device current when the batch was created
-    sim_batch() { stage_retain(); }
     ~sim_batch() {
-        stage_release();
         if (pool) rtl::pool_extra_free(pool);
         if (graph) cudaGraphExecDestroy(graph);
         if (pgraph) cudaGraphExecDestroy(pgraph);
@@ -396,6 +396,10 @@ int sim_load_netlist(const void* text, size_t len, const sim_config* cfg, sim_ne
         }
         h->mem_word_off.assign(1, 0);
         for (uint8_t lg : nl.mem_lg) h->mem_word_off.push_back(h->mem_word_off.back() + (1ULL << lg));
+        size_t words = nl.reg_w.size() < kStageBytes / 8 ? nl.reg_w.size() : 0;
+        for (uint8_t lg : nl.mem_lg)
+            if ((1ULL << lg) < kStageBytes / 8) words = std::max(words, size_t(1) << lg);
+        h->stage.bytes = (words + 1) * 8;
         sim_netlist_info& I = h->info;
         I.n_inputs = uint32_t(nl.in_w.size());
         I.n_regs = uint32_t(nl.reg_w.size());
@@ -1254,7 +1258,7 @@ int step_graph(sim_batch* b, uint64_t n) {
 // cycles of the 2k-op netlist and its registers: 84 -> 49 us).
 int read_back(sim_batch* b, uint32_t inst, int32_t mem, uint32_t n, uint64_t* out) {
     if (int rc = refuse_failed(b)) return rc;
-    Stage st;
+    Stage st(b->nl->stage);
     if (int rc = st.take()) return rc;
     CUDA_TRY(launch_read(b->stream, b->P, b->S, uint32_t(b->cycle & 1), inst, mem, n, st.p));
     CUDA_TRY(cudaStreamSynchronize(b->stream));

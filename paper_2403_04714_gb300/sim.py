@@ -184,7 +184,7 @@ def default_config(**kw) -> sim_config:
     return cfg
 
 
-SIM_COUNT_PLANS = 0
+SIM_COUNT_PLANS, SIM_COUNT_PINNED = 0, 1
 
 
 def debug_count(what: int) -> int:
