@@ -328,6 +328,11 @@ int sim_debug_skip_arrival(sim_batch *b, uint32_t timeout_ms);
 enum { SIM_COUNT_PLANS = 0, SIM_COUNT_PINNED, SIM_COUNT_KINDS };
 uint64_t sim_debug_count(int32_t what);
 
+/* Testing hook: the device form of one per-operation program (n words, as in
+ * the c_words table) into out (n words).  Errors: BADARG, STATE (a program
+ * that the interpreter could not run to its end). */
+int sim_debug_encode(const uint32_t *words, size_t n, uint32_t *out);
+
 /* Testing hook: the launch plan that the lane = instance bytecode of `groups`
  * x 32 instances gets on 1 / share of a GB300 (152 SMs), worked out without a
  * GPU: out = CTAs, warps per CTA, rounds of tasks, banded (0/1), shared memory

@@ -2006,7 +2006,57 @@ void encode_op(const DIns& d, bool second, uint32_t out[4]) {
 
 }  // namespace
 
-void encode_programs(Lowered& low) {
+int encode_program(const uint32_t* w, size_t words, uint32_t* e_words, uint32_t& e_tab, std::string& err) {
+    // the interpreter's loops rely on all of this: a run of operator or pair
+    // steps ends at a step of another kind, not at the program's end
+    const auto bad = [&](const char* what) {
+        err = std::string("internal error: compact program with ") + what;
+        return SIM_ERR_STATE;
+    };
+    const uint64_t nb = words ? w[0] : 0, tw = (nb + 4) & ~3ull;
+    if (!words || nb > 0xffff || tw > words) return bad("a step table of the wrong length");
+    uint64_t ni = 0;
+    for (uint32_t b = 0; b < nb; b++) {
+        const uint32_t e = w[1 + b], cnt = (e >> 16) & kStepCountMask;
+        const bool pair = e & kStepChain, generic = e & kStepGeneric;
+        if ((e & 0xffff) != ni) return bad("instructions out of order");
+        if (cnt == 0) return bad("an empty step");
+        if (pair ? cnt % 2 != 0 || cnt > 64 : cnt > (e & (kStepLeaf | kStepStore) ? kLeafStepMax : 32)) return bad("a step too wide");
+        if (b + 1 == nb && (pair || !generic)) return bad("operators in its last step");
+        ni += cnt;
+    }
+    if (tw + ni * 4 != words) return bad("instructions outside its steps");
+    memcpy(e_words, w, words * 4);
+    const DIns* ins = reinterpret_cast<const DIns*>(w + tw);
+    uint32_t *out = e_words + tw, *table = e_words + 1;
+    e_tab = uint32_t(tw / 4);
+    uint32_t ne = 0;                        // steps of the device form
+    for (uint32_t b = 0; b < nb; b++) {
+        const uint32_t e = w[1 + b], first = e & 0xffff, cnt = (e >> 16) & kStepCountMask;
+        const bool pair = e & kStepChain;
+        if (!pair && (e & kStepGeneric)) {
+            // register and mirror stores of neighbouring steps form wide store steps
+            bool stores = !(e & kStepLeaf);
+            for (uint32_t i = 0; i < cnt && stores; i++) stores = ins[first + i].op == D_STR || ins[first + i].op == D_STX;
+            const uint32_t last = ne ? table[ne - 1] : 0, have = (last >> 16) & kStepCountMask;
+            if (stores && (last & kStepStore) && have + cnt <= kLeafStepMax)
+                table[ne - 1] = (last & ~(kStepCountMask << 16)) | (have + cnt) << 16;
+            else
+                table[ne++] = e | (stores ? kStepStore : 0u);
+            continue;
+        }
+        // a lane's two operators side by side; step words hold the last lane
+        const uint32_t n = pair ? cnt / 2 : cnt;
+        for (uint32_t i = 0; i < cnt; i++)
+            encode_op(ins[first + i], i >= n, out + size_t(first + (pair ? i % n * 2 + i / n : i)) * 4);
+        table[ne++] = (e & ~(kStepCountMask << 16)) | (n - 1) << 16;
+    }
+    for (uint32_t b = ne; b < nb; b++) table[b] = 0;
+    e_words[0] = ne | uint32_t(tw / 4) << 16;
+    return SIM_OK;
+}
+
+int encode_programs(Lowered& low, std::string& err) {
     low.k_ins = low.b_ins;
     for (DIns& d : low.k_ins) {
         uint32_t kind = K_OTHER;
@@ -2022,39 +2072,12 @@ void encode_programs(Lowered& low) {
         }
         d.op = uint8_t(d.op | kind << 5);
     }
-    low.e_words = low.c_words;
+    low.e_words.assign(low.c_words.size(), 0);
     low.e_tab.assign(low.c_off.size(), 0);
-    for (size_t p = 0; p < low.c_off.size(); p++) {
-        const uint32_t* w = low.c_words.data() + low.c_off[p];
-        const uint32_t nb = w[0], tw = (nb + 4) & ~3u;
-        const DIns* ins = reinterpret_cast<const DIns*>(w + tw);
-        uint32_t* out = low.e_words.data() + low.c_off[p] + tw;
-        low.e_tab[p] = tw / 4;
-        uint32_t* table = low.e_words.data() + low.c_off[p] + 1;
-        uint32_t ne = 0;                        // steps of the device form
-        for (uint32_t b = 0; b < nb; b++) {
-            const uint32_t e = w[1 + b], first = e & 0xffff, cnt = (e >> 16) & kStepCountMask;
-            const bool pair = e & kStepChain;
-            if (!pair && (e & kStepGeneric)) {
-                // register and mirror stores of neighbouring steps form wide store steps
-                bool stores = !(e & kStepLeaf) && cnt > 0;
-                for (uint32_t i = 0; i < cnt && stores; i++) stores = ins[first + i].op == D_STR || ins[first + i].op == D_STX;
-                const uint32_t last = ne ? table[ne - 1] : 0, have = (last >> 16) & kStepCountMask;
-                if (stores && (last & kStepStore) && have + cnt <= kLeafStepMax)
-                    table[ne - 1] = (last & ~(kStepCountMask << 16)) | (have + cnt) << 16;
-                else
-                    table[ne++] = e | (stores ? kStepStore : 0u);
-                continue;
-            }
-            // a lane's two operators side by side; step words hold the last lane
-            const uint32_t n = pair ? cnt / 2 : cnt;
-            for (uint32_t i = 0; i < cnt; i++)
-                encode_op(ins[first + i], i >= n, out + size_t(first + (pair ? i % n * 2 + i / n : i)) * 4);
-            table[ne++] = (e & ~(kStepCountMask << 16)) | (n - 1) << 16;
-        }
-        for (uint32_t b = ne; b < nb; b++) table[b] = 0;
-        low.e_words[low.c_off[p]] = ne | (tw / 4) << 16;
-    }
+    for (size_t p = 0; p < low.c_off.size(); p++)
+        if (int rc = encode_program(low.c_words.data() + low.c_off[p], low.c_size[p], low.e_words.data() + low.c_off[p], low.e_tab[p], err))
+            return rc;
+    return SIM_OK;
 }
 
 // ---------------------------------------------------------------------------

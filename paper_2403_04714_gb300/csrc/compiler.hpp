@@ -125,7 +125,11 @@ int lower(const Netlist& nl, const Partition& part, Lowered& out, std::string& e
 // the instruction count; neighbouring steps of stores merged into wide store
 // steps; everything else as it is.  Word 0: steps | 16-byte units before the
 // instructions << 16.
-void encode_programs(Lowered& low);
+// SIM_ERR_STATE if a program is not one that the interpreter's loops end on:
+// an empty or too wide step, or a last step of operators.
+int encode_programs(Lowered& low, std::string& err);
+// One of them: `words` words from w to e_words, which is as long.
+int encode_program(const uint32_t* w, size_t words, uint32_t* e_words, uint32_t& e_tab, std::string& err);
 
 // Cluster exchange.  Processes are placed on a grid of thread-block
 // clusters (C CTAs of W warps, one process per warp) so that producers and

@@ -378,7 +378,8 @@ int sim_load_netlist(const void* text, size_t len, const sim_config* cfg, sim_ne
             rc = lower_clusters(h->nl, h->part, C, W, h->low, h->cplan, err, h->cfg.chain < 2);
             if (rc) return set_err(rc, err);
         }
-        encode_programs(h->low);
+        rc = encode_programs(h->low, err);
+        if (rc) return set_err(rc, err);
         auto descending = [](const auto& key) {
             std::vector<uint32_t> v(key.size());
             for (size_t p = 0; p < v.size(); p++) v[p] = uint32_t(p);
@@ -1781,6 +1782,14 @@ int sim_debug_skip_arrival(sim_batch* b, uint32_t timeout_ms) {
 }
 
 uint64_t sim_debug_count(int32_t what) { return what >= 0 && what < SIM_COUNT_KINDS ? g_counts[what].load() : 0; }
+
+int sim_debug_encode(const uint32_t* words, size_t n, uint32_t* out) {
+    if (!words || !out) return set_err(SIM_ERR_BADARG, "null argument");
+    std::string err;
+    uint32_t tab = 0;
+    const int rc = encode_program(words, n, out, tab, err);
+    return rc ? set_err(rc, err) : SIM_OK;
+}
 
 int sim_debug_lane_plan(const sim_netlist* nl, uint32_t groups, uint32_t share, int32_t per_cycle, uint64_t* out) {
     if (!nl || !groups || !out || nl->low.b_slots.empty()) return set_err(SIM_ERR_BADARG, "bad argument");

@@ -95,6 +95,7 @@ EXPORTS = {
     "sim_launch_info": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
     "sim_debug_skip_arrival": (C.c_int, [C.c_void_p, C.c_uint32]),
     "sim_debug_count": (C.c_uint64, [C.c_int32]),
+    "sim_debug_encode": (C.c_int, [C.c_void_p, C.c_size_t, C.c_void_p]),
     "sim_debug_lane_plan": (C.c_int, [C.c_void_p, C.c_uint32, C.c_uint32, C.c_int32, C.c_void_p]),
     "sim_last_error": (C.c_char_p, []),
     "sim_netlist_table": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p]),
@@ -197,6 +198,14 @@ def measure_int_peak(iters: int = 4096) -> float:
     v = C.c_double()
     _check(lib().sim_measure_int_peak(iters, C.byref(v)))
     return v.value
+
+
+def debug_encode(words: np.ndarray) -> np.ndarray:
+    """sim_debug_encode: the device form of one per-operation program."""
+    words = np.ascontiguousarray(words, dtype=np.uint32)
+    out = np.zeros_like(words)
+    _check(lib().sim_debug_encode(words.ctypes.data, len(words), out.ctypes.data))
+    return out
 
 
 class Netlist:
