@@ -203,6 +203,10 @@ int sim_netlist_compile_generated(sim_netlist *nl, int32_t mode, double *seconds
  *  20 {CTAs per cluster, warps per CTA, grid CTAs, mirror entries per CTA, cross-process register reads
  *      inside a cluster, reads across clusters} (u64 x 6)
  *  21 log2 of the depth of each memory (u8)
+ *  Programs as the device runs them (layouts in abi_device.h):
+ *  22 per-operation programs (u32, placed as in 15 and 16)
+ *  23 16-byte units before the instructions of each (u32)
+ *  24 instructions of table 3 with their kind above the opcode (16 bytes)
  * Errors: BADARG. */
 int sim_netlist_table(const sim_netlist *nl, int32_t which, void *out, size_t *bytes);
 

@@ -495,6 +495,9 @@ int sim_netlist_table(const sim_netlist* nl, int32_t which, void* out, size_t* b
         break;
     }
     case 21: pick(nl->nl.mem_lg); break;
+    case 22: pick(L.e_words); break;
+    case 23: pick(L.e_tab); break;
+    case 24: pick(L.k_ins); break;
     default: return set_err(SIM_ERR_BADARG, "unknown table");
     }
     if (out) memcpy(out, src, std::min(n, *bytes));

@@ -136,7 +136,8 @@ TABLES = {"s_ins": (0, None), "s_off": (1, np.uint32), "s_len": (2, np.uint32), 
           "reg_cls": (10, np.uint8), "reg_idx": (11, np.uint32), "s_slots": (12, np.uint32),
           "b_slots": (13, np.uint32), "c_words": (14, np.uint32), "c_off": (15, np.uint32),
           "c_size": (16, np.uint32), "warp_proc": (17, np.uint32), "mir_off": (18, np.uint32),
-          "mir_reg": (19, np.uint32), "cluster_plan": (20, np.uint64), "mem_lg": (21, np.uint8)}
+          "mir_reg": (19, np.uint32), "cluster_plan": (20, np.uint64), "mem_lg": (21, np.uint8),
+          "e_words": (22, np.uint32), "e_tab": (23, np.uint32), "k_ins": (24, None)}
 # one 16-byte instruction of the device bytecode
 DINS = np.dtype([("op", np.uint8), ("w", np.uint8), ("dst", np.uint16), ("a", np.uint16), ("b", np.uint16),
                  ("c", np.uint16), ("x", np.uint16), ("imm", np.uint32)])
