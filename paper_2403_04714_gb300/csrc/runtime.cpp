@@ -1864,7 +1864,11 @@ size_t pool_footprint(const sim_netlist* h, uint32_t capacity) {
     // memories, write records, held inputs (value + flag) and, with generated
     // code, the input values of two cycles
     per += h->mem_word_off.back() * 8 + nl.wports.size() * 32 + nl.in_w.size() * (9 + 16) + nl.mem_lg.size() * 8 + 40;
-    uint64_t prog = (h->low.s_ins.size() + h->low.b_ins.size()) * 16 + h->low.c_words.size() * 4;
+    // a pool has the lane = instance program only: the bytecode with its four
+    // tables of a word per process, or generated code, about five times as long
+    // (200k-op netlist: 3.4 MB of bytecode, a module of 15.2 MB)
+    const bool gen = h->cfg.lowering == SIM_LOWER_GENERATED;
+    const uint64_t prog = h->low.b_ins.size() * 16 * (gen ? 5 : 1) + h->part.procs.size() * 16;
     return size_t(per * I + prog + 2 * h->mem_word_off.back() * 8);
 }
 
