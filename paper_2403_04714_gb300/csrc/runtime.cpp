@@ -1256,12 +1256,26 @@ int step_graph(sim_batch* b, uint64_t n) {
     return SIM_OK;
 }
 
+// The batch's device, current while kernels gather for a read or a checkpoint:
+// a copy takes any current device, a launch only its stream's.
+struct OnDevice {
+    int before = -1;
+    explicit OnDevice(int device) {
+        int cur = device;
+        if (cudaGetDevice(&cur) == cudaSuccess && cur != device && cudaSetDevice(device) == cudaSuccess) before = cur;
+    }
+    ~OnDevice() {
+        if (before >= 0) cudaSetDevice(before);
+    }
+};
+
 // One instance's registers (mem < 0) or the n words of a memory: a kernel writes
 // them and the error word to pinned memory, one wait in place of a copy of the
 // error word and three strided copies with waits of their own (a step of 8
 // cycles of the 2k-op netlist and its registers: 84 -> 49 us).
 int read_back(sim_batch* b, uint32_t inst, int32_t mem, uint32_t n, uint64_t* out) {
     if (int rc = refuse_failed(b)) return rc;
+    OnDevice on(b->device);
     Stage st(b->nl->stage);
     if (int rc = st.take()) return rc;
     CUDA_TRY(launch_read(b->stream, b->P, b->S, uint32_t(b->cycle & 1), inst, mem, n, st.p));
@@ -1668,6 +1682,7 @@ int sim_save(sim_batch* b, void** blob, size_t* len) {
     // registers in [register][instance] order whatever the kernels' layout
     uint32_t par = uint32_t(b->cycle & 1);
     int rc = sim_sync(b);
+    OnDevice on(b->device);
     if (!rc && S.pack == 32) {
         if (launch_retile(b->stream, S, par, false) != cudaSuccess) rc = set_err(SIM_ERR_CUDA, "checkpoint kernel failed");
         par ^= 1;
@@ -1725,7 +1740,10 @@ int sim_restore(sim_batch* b, const void* blob, size_t len) {
     };
     if (!h2d(S.bits[par], nb) || !h2d(S.w32[par], n32) || !h2d(S.w64[par], n64) || !h2d(S.mem, nm) || !h2d(S.mem_dig, nmd))
         return set_err(SIM_ERR_CUDA, "restore copy failed");
-    if (tiled) CUDA_TRY(launch_retile(b->stream, S, par ^ 1u, true));
+    if (tiled) {
+        OnDevice on(b->device);
+        CUDA_TRY(launch_retile(b->stream, S, par ^ 1u, true));
+    }
     if (nh) {
         memcpy(b->h_hold_val.data(), q, nh * 8);
         q += nh * 8;
