@@ -165,20 +165,23 @@ struct Stage {
     StagePool& pool;
     uint64_t* p = nullptr;
     explicit Stage(StagePool& s) : pool(s) {}
-    int take() {
+    bool take() {
         {
             std::lock_guard<std::mutex> g(pool.mu);
             if (!pool.kept.empty()) {
                 p = static_cast<uint64_t*>(pool.kept.back());
                 pool.kept.pop_back();
-                return SIM_OK;
+                return true;
             }
         }
         void* v = nullptr;
-        CUDA_TRY(cudaHostAlloc(&v, pool.bytes, cudaHostAllocPortable | cudaHostAllocMapped));
+        if (cudaHostAlloc(&v, pool.bytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
         g_counts[SIM_COUNT_PINNED]++;
         p = static_cast<uint64_t*>(v);
-        return SIM_OK;
+        return true;
     }
     ~Stage() {
         if (!p) return;
@@ -1272,16 +1275,19 @@ struct OnDevice {
 // One instance's registers (mem < 0) or the n words of a memory: a kernel writes
 // them and the error word to pinned memory, one wait in place of a copy of the
 // error word and three strided copies with waits of their own (a step of 8
-// cycles of the 2k-op netlist and its registers: 84 -> 49 us).
-int read_back(sim_batch* b, uint32_t inst, int32_t mem, uint32_t n, uint64_t* out) {
+// cycles of the 2k-op netlist and its registers: 84 -> 49 us).  kNotRead where
+// the read-back is too long for the pinned buffer or there is none to be had:
+// the caller copies it then.
+constexpr int kNotRead = 1;
+int read_back(sim_batch* b, uint32_t inst, int32_t mem, size_t n, uint64_t* out) {
     if (int rc = refuse_failed(b)) return rc;
     OnDevice on(b->device);
     Stage st(b->nl->stage);
-    if (int rc = st.take()) return rc;
-    CUDA_TRY(launch_read(b->stream, b->P, b->S, uint32_t(b->cycle & 1), inst, mem, n, st.p));
+    if (n >= kStageBytes / 8 || !st.take()) return kNotRead;
+    CUDA_TRY(launch_read(b->stream, b->P, b->S, uint32_t(b->cycle & 1), inst, mem, uint32_t(n), st.p));
     CUDA_TRY(cudaStreamSynchronize(b->stream));
     if (st.p[0]) return check_err(b);
-    memcpy(out, st.p + 1, size_t(n) * 8);
+    memcpy(out, st.p + 1, n * 8);
     return SIM_OK;
 }
 
@@ -1563,7 +1569,7 @@ int sim_peek_mems(sim_batch* b, uint32_t inst, uint32_t mem, uint64_t* out) {
     const Netlist& nl = b->nl->nl;
     if (!out || mem >= nl.mem_lg.size()) return set_err(SIM_ERR_BADARG, "bad argument");
     const size_t depth = size_t(1) << nl.mem_lg[mem];
-    if (depth < kStageBytes / 8) return read_back(b, inst, int32_t(mem), uint32_t(depth), out);
+    if ((rc = read_back(b, inst, int32_t(mem), depth, out)) != kNotRead) return rc;
     rc = sim_sync(b);
     if (rc) return rc;
     // instance-minor layout: word a of instance inst is at (base + a) * I + inst
@@ -1578,7 +1584,7 @@ int sim_peek_regs(sim_batch* b, uint32_t inst, uint64_t* out) {
     if (rc) return rc;
     if (!out) return set_err(SIM_ERR_BADARG, "null output");
     const RegLayout& L = b->nl->layout;
-    if (L.cls.size() < kStageBytes / 8) return read_back(b, inst, -1, uint32_t(L.cls.size()), out);
+    if ((rc = read_back(b, inst, -1, L.cls.size(), out)) != kNotRead) return rc;
     rc = sim_sync(b);
     if (rc) return rc;
     const DevState& S = b->S;

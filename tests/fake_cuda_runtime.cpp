@@ -1,7 +1,7 @@
 // Two pretended GPUs for CPU tests, preloaded in front of the CUDA runtime:
 // device memory is host memory, kernels do nothing, and a launch on a stream of
 // another device than the current one fails, as it does on hardware (copies and
-// waits do not).
+// waits do not).  FAKE_CUDA_NO_PINNED in the environment: no pinned memory.
 #include <cuda_runtime_api.h>
 
 #include <cstdlib>
@@ -33,7 +33,10 @@ cudaError_t cudaGetLastError() {
 }
 cudaError_t cudaMalloc(void** p, size_t n) { return *p = calloc(n ? n : 1, 1), cudaSuccess; }
 cudaError_t cudaFree(void* p) { return free(p), cudaSuccess; }
-cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return *p = calloc(n, 1), cudaSuccess; }
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) {
+    if (getenv("FAKE_CUDA_NO_PINNED")) return g_last = cudaErrorMemoryAllocation;
+    return *p = calloc(n, 1), cudaSuccess;
+}
 cudaError_t cudaFreeHost(void* p) { return free(p), cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { return memmove(d, s, n), cudaSuccess; }
 cudaError_t cudaMemcpy2DAsync(void* d, size_t dp, const void* s, size_t sp, size_t w, size_t h, cudaMemcpyKind, cudaStream_t) {

@@ -1,0 +1,82 @@
+"""Reads and checkpoints on the host side (CPU only, behind a stand-in for the
+CUDA runtime with two pretended GPUs): while another device than the batch's is
+current, and without pinned memory.  For the caller they are plain copies, which
+need neither."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+
+PROGRAM = """
+import ctypes
+from paper_2403_04714_gb300 import netgen, sim
+
+fake = ctypes.CDLL(None)
+def current():
+    d = ctypes.c_int()
+    fake.cudaGetDevice(ctypes.byref(d))
+    return d.value
+
+text = netgen.gen_flat(5, n_ops=900, n_regs=60, depth=12, n_inputs=4, rams=((3, 64),)).to_text()
+for n_inst in (1, 33):
+    fake.cudaSetDevice(0)
+    b = sim.Batch(sim.Netlist(text), n_inst)
+    b.step(3)
+    for device in (0, 1):
+        fake.cudaSetDevice(device)
+        b.regs(n_inst - 1)
+        b.mem_all(n_inst - 1, 0)
+        b.restore(b.save())
+        b.peek_reg(0, 1)
+        assert current() == device
+    b.close()
+print("done")
+"""
+
+
+NO_PINNED = """
+from paper_2403_04714_gb300 import netgen, sim
+
+text = netgen.gen_flat(5, n_ops=900, n_regs=60, depth=12, n_inputs=4, rams=((3, 64),)).to_text()
+nl = sim.Netlist(text)
+init = [int(l.split()[2]) for l in text.splitlines() if l.startswith("reg ")]
+width = [int(l.split()[1]) for l in text.splitlines() if l.startswith("reg ")]
+assert any(init) and {1, 32, 64} <= set(width)
+for n_inst in (1, 70):
+    b = sim.Batch(nl, n_inst)
+    b.step(2)                                   # pretended kernels change nothing
+    for i in {0, n_inst // 2, n_inst - 1}:
+        assert list(b.regs(i)) == init
+        want = [hash((i, r)) % 2 ** w for r, w in enumerate(width)]
+        for r, v in enumerate(want):
+            b.poke_reg(i, r, v)
+        words = [hash((i, a)) % 2 ** 64 for a in range(8)]
+        for a, v in enumerate(words):
+            b.poke_mem(i, 0, a, v)
+        assert list(b.regs(i)) == want and list(b.mem_all(i, 0)) == words
+print("done")
+"""
+
+
+def run(program, tmp_path, **env):
+    if not shutil.which("g++") or not os.path.exists(f"{CUDA}/include/cuda_runtime_api.h"):
+        pytest.skip("needs g++ and the CUDA headers")
+    so = str(tmp_path / "fake_cuda_runtime.so")
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", f"-I{CUDA}/include", "-o", so, os.path.join(HERE, "fake_cuda_runtime.cpp")],
+                   check=True)
+    r = subprocess.run([sys.executable, "-c", program], cwd=os.path.dirname(HERE), capture_output=True, text=True, timeout=120,
+                       env={**os.environ, "LD_PRELOAD": so, **env})
+    assert r.returncode == 0 and "done" in r.stdout, r.stdout + r.stderr
+
+
+def test_reads_and_checkpoints_take_any_current_device(tmp_path):
+    run(PROGRAM, tmp_path)
+
+
+def test_reads_without_pinned_memory(tmp_path):
+    run(NO_PINNED, tmp_path, FAKE_CUDA_NO_PINNED="1")
