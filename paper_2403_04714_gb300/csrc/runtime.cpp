@@ -729,7 +729,9 @@ int plan_lane_inst(sim_batch* b, uint32_t share) {
 // resident; the CTA size with the fewest instances per warp (then the fewest
 // warps per SM).  One warp per process ran the instances one after the other:
 // the 2k-op netlist x 8, 70 processes, took 25.8 us a cycle on 18 of the SMs,
-// and 4.3 us with a warp for each of the 560 tasks.
+// and 4.3 us with a warp for each of the 560 tasks.  Called with the plan of
+// one warp per process, or without resident programs, in b; that stays where it
+// is the better one.
 int plan_replicas(sim_batch* b, size_t slot_bytes) {
     const Lowered& L = b->nl->low;
     const uint32_t n_proc = uint32_t(L.c_size.size());
@@ -753,6 +755,18 @@ int plan_replicas(sim_batch* b, size_t slot_bytes) {
         if (share < best_share) best_share = share, best_warps = uint32_t(w), best_smem = smem, best_occ = occ;
     }
     if (!best_warps) return SIM_OK;
+    // Few processes with programs of which only some hundred fit at a time: the
+    // plan without resident programs has a warp for every task instead, in
+    // fewer rounds.  One of its rounds took 1.7 to 2 times an instance of a
+    // resident program at up to 8 warps per SM, 2.3 to 2.6 at 13 and 3.8 at 32;
+    // the line is (24 + warps per SM) / 16 (200k-op netlist in 30 processes,
+    // us a cycle resident against not: 8 instances 78 and 68, 16 147 and 71, 64
+    // 458 and 93, 200 1,432 and 336; in 152 processes 200 instances 329 and 337)
+    if (b->prog_words == 0) {
+        const uint64_t total = uint64_t(b->grid) * b->warps;
+        const uint64_t rounds = (b->n_tasks + total - 1) / total, per_sm = (total + sms - 1) / sms;
+        if (best_share * 16ull > rounds * (24 + per_sm)) return SIM_OK;
+    }
     b->replicas = (b->I + best_share - 1) / best_share;       // no more than that share needs
     b->warps = int(best_warps);
     b->threads = b->warps * 32;
@@ -763,38 +777,18 @@ int plan_replicas(sim_batch* b, size_t slot_bytes) {
     return SIM_OK;
 }
 
-// Choose warps per CTA and grid for a batch (both lane mappings).  LANE_OP
-// keeps each warp's programs resident in shared memory when they fit.
-int plan_launch(sim_batch* b) {
+// A warp per process, its program in shared memory when it fits (the instances
+// one after the other), else a warp per task with programs in global memory.
+int plan_one_warp(sim_batch* b, int warps, size_t slot_bytes) {
     const Lowered& L = b->nl->low;
     const int sms = sm_count();
     const size_t smem_cap = smem_limit();
     const uint32_t n_proc = uint32_t(b->nl->part.procs.size());
-    if (b->mode == SIM_MODE_LANE_INST) {
-        b->slot_words = L.max_b_slots * 32 + kBlockWords;
-        b->n_tasks = n_proc * (b->I / 32);
-    } else {
-        b->slot_words = (L.max_s_slots + 2) & ~1u;   // at least one spare slot (the operator steps' dummy)
-        b->n_tasks = n_proc * b->I;
-    }
-    size_t slot_bytes = size_t(b->slot_words) * 8;
-    if (slot_bytes > smem_cap)
-        return set_err(SIM_ERR_CAPACITY, "a process needs " + std::to_string(slot_bytes) +
-                                             " bytes of value slots per warp (limit " + std::to_string(smem_cap) + ")");
-    int warps = b->cfg.warps_per_cta ? int(b->cfg.warps_per_cta) : 8;
-    if (!b->cfg.warps_per_cta && b->mode == SIM_MODE_LANE_OP)   // one process per warp, one CTA per SM
-        warps = int(std::min<uint64_t>(16, std::max<uint64_t>(1, (uint64_t(n_proc) * b->I + sms - 1) / sms)));
-    if (b->mode == SIM_MODE_LANE_INST && b->proc_major && !b->wave_groups && n_proc) return plan_lane_inst(b, 1);
-    while (warps > 1 && size_t(warps) * slot_bytes > smem_cap) warps /= 2;
     b->warps = warps;
     b->threads = warps * 32;
     b->prog_words = 0;
-    int occ = 0;
     b->replicas = 1;
-    if (b->mode == SIM_MODE_LANE_OP && b->I > 1 && n_proc) {
-        int rc = plan_replicas(b, slot_bytes);
-        if (rc || b->replicas > 1) return rc;
-    }
+    int occ = 0;
     if (b->mode == SIM_MODE_LANE_OP) {
         // one process per warp when the grid allows it; re-plan with the
         // smaller grid if the resident programs lower occupancy
@@ -825,6 +819,34 @@ int plan_launch(sim_batch* b) {
     int need = int((b->n_tasks + warps - 1) / warps);
     b->grid = std::max(1, std::min(need, b->max_grid));
     return SIM_OK;
+}
+
+// Choose warps per CTA and grid for a batch (both lane mappings).  LANE_OP
+// keeps each warp's programs resident in shared memory when they fit.
+int plan_launch(sim_batch* b) {
+    const Lowered& L = b->nl->low;
+    const int sms = sm_count();
+    const size_t smem_cap = smem_limit();
+    const uint32_t n_proc = uint32_t(b->nl->part.procs.size());
+    if (b->mode == SIM_MODE_LANE_INST) {
+        b->slot_words = L.max_b_slots * 32 + kBlockWords;
+        b->n_tasks = n_proc * (b->I / 32);
+    } else {
+        b->slot_words = (L.max_s_slots + 2) & ~1u;   // at least one spare slot (the operator steps' dummy)
+        b->n_tasks = n_proc * b->I;
+    }
+    size_t slot_bytes = size_t(b->slot_words) * 8;
+    if (slot_bytes > smem_cap)
+        return set_err(SIM_ERR_CAPACITY, "a process needs " + std::to_string(slot_bytes) +
+                                             " bytes of value slots per warp (limit " + std::to_string(smem_cap) + ")");
+    int warps = b->cfg.warps_per_cta ? int(b->cfg.warps_per_cta) : 8;
+    if (!b->cfg.warps_per_cta && b->mode == SIM_MODE_LANE_OP)   // one process per warp, one CTA per SM
+        warps = int(std::min<uint64_t>(16, std::max<uint64_t>(1, (uint64_t(n_proc) * b->I + sms - 1) / sms)));
+    if (b->mode == SIM_MODE_LANE_INST && b->proc_major && !b->wave_groups && n_proc) return plan_lane_inst(b, 1);
+    while (warps > 1 && size_t(warps) * slot_bytes > smem_cap) warps /= 2;
+    const int rc = plan_one_warp(b, warps, slot_bytes);
+    if (rc || b->mode != SIM_MODE_LANE_OP || b->I == 1 || !n_proc) return rc;
+    return plan_replicas(b, slot_bytes);
 }
 
 int upload_program(sim_batch* b) {

@@ -1,7 +1,7 @@
-"""Reads and checkpoints on the host side (CPU only, behind a stand-in for the
-CUDA runtime with two pretended GPUs): while another device than the batch's is
-current, and without pinned memory.  For the caller they are plain copies, which
-need neither."""
+"""Host calls (CPU only, behind a stand-in for the CUDA runtime with two pretended
+GPUs).  Reads and checkpoints while another device than the batch's is current,
+and without pinned memory: for the caller they are plain copies, which need
+neither.  Launch plans of several instances with lane = operation."""
 import os
 import shutil
 import subprocess
@@ -62,6 +62,31 @@ for n_inst in (1, 70):
 print("done")
 """
 
+PLANS = """
+from paper_2403_04714_gb300 import netgen, sim
+
+def plan(nl, n_inst):
+    b = sim.Batch(nl, n_inst)
+    i = b.launch_info()
+    b.close()
+    return i["ctas"] * i["warps_per_cta"], i["tasks_per_cycle"]
+
+# few large processes: a warp for every task, not one for several instances in turn
+text = open(netgen.cached_netlist("mid")).read()
+few = sim.Netlist(text, mode="lane_op", target_processes=30)
+for n in (8, 16, 31, 64):
+    warps, tasks = plan(few, n)
+    assert tasks == 30 * n and warps >= tasks, (n, warps, tasks)
+warps, tasks = plan(few, 200)
+assert warps >= 1216, warps
+# resident programs where they are the better ones
+assert plan(few, 5)[0] == 150
+some = sim.Netlist(text, mode="lane_op", target_processes=152)
+assert plan(some, 16)[0] == 1216
+assert plan(sim.Netlist(open(netgen.cached_netlist("tiny")).read(), mode="lane_op"), 8)[0] == 560
+print("done")
+"""
+
 
 def run(program, tmp_path, **env):
     if not shutil.which("g++") or not os.path.exists(f"{CUDA}/include/cuda_runtime_api.h"):
@@ -80,3 +105,7 @@ def test_reads_and_checkpoints_take_any_current_device(tmp_path):
 
 def test_reads_without_pinned_memory(tmp_path):
     run(NO_PINNED, tmp_path, FAKE_CUDA_NO_PINNED="1")
+
+
+def test_plans_of_several_instances(tmp_path):
+    run(PLANS, tmp_path)
