@@ -42,6 +42,8 @@ __device__ __forceinline__ void red_release_add(unsigned long long* p, unsigned 
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+constexpr uint32_t kQuickPollCtas = 608;     // four per SM
+
 // Grid-wide barrier on one monotonic 64-bit arrival counter (zeroed before
 // each launch): barrier number g of the launch is complete once the counter
 // reaches (g+1) x gridDim.x.  Each CTA adds its arrival with a release
@@ -51,8 +53,11 @@ __device__ __forceinline__ void red_release_add(unsigned long long* p, unsigned 
 // publish a generation word, so the last arrival releases everyone directly.
 // The error word and the clock are read after every sixteenth poll: after each
 // one they doubled the time between polls (2k-op netlist 3.83 -> 3.76 us a
-// cycle, 200k-op netlist 9.11 -> 9.05).  A flag per CTA, polled by every other
-// CTA's warp, measured 3 us slower a cycle.
+// cycle, 200k-op netlist 9.11 -> 9.05).  Above kQuickPollCtas CTAs that time is
+// wanted: their polls crowd out the arrivals on the same word (2k-op netlist,
+// generated code x 2,500 in 4,864 CTAs 22.8 -> 19.4 us a cycle, 1,216 CTAs 7.26 ->
+// 6.58, 760 CTAs 5.35 -> 5.14; 608 and fewer are the better without it).  A flag
+// per CTA, polled by every other CTA's warp, measured 3 us slower a cycle.
 // Every wait is bounded: past `timeout_ns`, or once another CTA has recorded
 // an error, the CTA records SIM_ERR_TIMEOUT (first error wins) and returns
 // false.  With `rec` set, thread 0 stores the time the whole CTA arrived
@@ -67,9 +72,10 @@ static __device__ bool grid_barrier(uint32_t* bar, uint32_t& gen, uint64_t timeo
         unsigned long long* count = reinterpret_cast<unsigned long long*>(bar);
         const unsigned long long target = (unsigned long long)(gen + 1) * gridDim.x;
         if (!skip) red_release_add(count, 1ull);
+        const uint32_t quick = gridDim.x <= kQuickPollCtas ? 15u : 0u;
         uint64_t start = 0;
         for (uint32_t polls = 1; ld_acquire_u64(count) < target; polls++) {
-            if (polls & 15u) continue;
+            if (polls & quick) continue;
             const uint64_t now = globaltimer_ns();
             if (!start) start = now;
             if (ld_volatile(err) != 0) { ok = 0; break; }
