@@ -575,6 +575,17 @@ int plan_grid_gen(sim_batch* b, uint32_t share) {
     b->max_grid = occ * sms;
     const int need = int((b->n_tasks + b->warps - 1) / b->warps);
     b->grid = std::max(1, std::min(need, std::max(1, b->max_grid / int(std::max(1u, share)))));
+    // CTAs of up to four warps: no more of them than the rounds need, whose
+    // last one is full then.  Their number is what the grid barrier costs (2k-op
+    // netlist x 2,500, us a cycle: one warp, 4,864 CTAs 19.1, 2,765 CTAs 14.3; four
+    // warps, 1,216 6.7, 692 5.4; 20k-op netlist x 700, one warp, 4,864 34.7, 3,344
+    // 28.9; 200k-op netlist x 700, four warps, 1,216 49.7, 836 45.4).  With six and
+    // more the warps in flight count for as much (20k-op netlist x 2,500, six
+    // warps: 760 CTAs 18.4, 668 20.2).
+    if (b->warps <= 4) {
+        const int rounds = (need + b->grid - 1) / b->grid;
+        b->grid = (need + rounds - 1) / rounds;
+    }
     return SIM_OK;
 }
 

@@ -1,7 +1,8 @@
 """Host calls (CPU only, behind a stand-in for the CUDA runtime with two pretended
 GPUs).  Reads and checkpoints while another device than the batch's is current,
 and without pinned memory: for the caller they are plain copies, which need
-neither.  Launch plans of several instances with lane = operation."""
+neither.  Launch plans of several instances with lane = operation, and of
+generated code."""
 import os
 import shutil
 import subprocess
@@ -87,6 +88,24 @@ assert plan(sim.Netlist(open(netgen.cached_netlist("tiny")).read(), mode="lane_o
 print("done")
 """
 
+GENERATED = """
+from paper_2403_04714_gb300 import netgen, sim
+
+text = open(netgen.cached_netlist("tiny")).read()
+for warps in (1, 2, 3, 4, 6, 8):
+    nl = sim.Netlist(text, mode="lane_inst", lowering="generated", warps_per_cta=warps)
+    for n in (1, 700, 2500, 4096, 9999):
+        b = sim.Batch(nl, n)
+        i = b.launch_info()
+        assert i["warps_per_cta"] == warps
+        need = -(-i["tasks_per_cycle"] // warps)
+        most = 32 // warps * 152
+        rounds = -(-need // most)
+        assert i["ctas"] == (-(-need // rounds) if warps <= 4 else min(need, most)), (warps, n, i)
+        b.close()
+print("done")
+"""
+
 
 def run(program, tmp_path, **env):
     if not shutil.which("g++") or not os.path.exists(f"{CUDA}/include/cuda_runtime_api.h"):
@@ -109,3 +128,7 @@ def test_reads_without_pinned_memory(tmp_path):
 
 def test_plans_of_several_instances(tmp_path):
     run(PLANS, tmp_path)
+
+
+def test_plans_of_generated_code(tmp_path):
+    run(GENERATED, tmp_path)
