@@ -14,9 +14,10 @@ struct GenUnit {
 };
 
 // CUDA sources for every process (in n_chunks units) plus the dispatcher and
-// one kernel for lane mapping `mode`: rtl_gen_d1 with the per-cycle digest
+// the kernels for lane mapping `mode`: rtl_gen_d1 with the per-cycle digest
 // code in every process function, or rtl_gen_d0 without any (its process
-// functions are that much shorter, which the instruction caches feel).
+// functions are that much shorter, which the instruction caches feel); and
+// rtl_cyc_d1 or rtl_cyc_d0 for launches of one cycle.
 int gen_cuda(const Netlist& nl, const Partition& part, int mode, bool digest, int n_chunks, std::vector<GenUnit>& out,
              std::string& err);
 void gen_process(const Netlist& nl, const Partition& part, const RegLayout& L, size_t p, int mode, bool digest,
@@ -26,6 +27,7 @@ void gen_process(const Netlist& nl, const Partition& part, const RegLayout& L, s
 struct GenModule {
     cudaLibrary_t lib = nullptr;
     cudaKernel_t kernel = nullptr;                 // rtl_gen_d0 or rtl_gen_d1
+    cudaKernel_t cycle_kernel = nullptr;           // rtl_cyc_d0 or rtl_cyc_d1, launches of one cycle
     double compile_seconds = 0;
     bool cached = false;
 };

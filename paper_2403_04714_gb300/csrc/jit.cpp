@@ -184,6 +184,7 @@ int jit_load(const std::vector<char>& linked, bool digest, GenModule& out, std::
         return SIM_ERR_CUDA;
     }
     e = cudaLibraryGetKernel(&out.kernel, out.lib, digest ? "rtl_gen_d1" : "rtl_gen_d0");
+    if (e == cudaSuccess) e = cudaLibraryGetKernel(&out.cycle_kernel, out.lib, digest ? "rtl_cyc_d1" : "rtl_cyc_d0");
     if (e != cudaSuccess) {
         err = std::string("cudaLibraryGetKernel: ") + cudaGetErrorString(e);
         cudaLibraryUnload(out.lib);
@@ -196,7 +197,7 @@ int jit_load(const std::vector<char>& linked, bool digest, GenModule& out, std::
 void jit_unload(GenModule& m) {
     if (m.lib) cudaLibraryUnload(m.lib);
     m.lib = nullptr;
-    m.kernel = nullptr;
+    m.kernel = m.cycle_kernel = nullptr;
 }
 
 }  // namespace rtl

@@ -226,6 +226,7 @@ struct sim_batch {
     rtl::PoolExtra* pool = nullptr;        // set for server pools
     bool generated = false;                // processes run as generated CUDA
     const void* gen_kernel[2] = {nullptr, nullptr};
+    const void* cycle_kernel[2] = {nullptr, nullptr};      // the same for launches of one cycle
     DevState S_uploaded{};
     cudaStream_t stream = nullptr;
     int mode = SIM_MODE_LANE_OP;
@@ -613,7 +614,7 @@ cudaError_t launch_any(sim_batch* b, bool cooperative, int grid, const LaunchArg
         return launch_cycles_cl(b->S.ring_cap > 0, grid, b->threads, b->smem, b->nl->cplan.C, b->stream, b->P, b->S, A);
     if (!b->generated)
         return launch_cycles(b->mode, b->S.ring_cap > 0, cooperative, grid, b->threads, b->smem, b->stream, b->P, b->S, A);
-    const void* f = b->gen_kernel[b->S.ring_cap > 0 ? 1 : 0];
+    const void* f = (A.grid_sync ? b->gen_kernel : b->cycle_kernel)[b->S.ring_cap > 0 ? 1 : 0];
     const DevProg* Pd = b->P_dev.as<DevProg>();
     const DevState* Sd = b->S_dev.as<DevState>();
     LaunchArgs a = A;
@@ -1406,6 +1407,7 @@ int create_instances(sim_netlist* nl, const sim_config& cfg, uint32_t n_inst, ui
             if ((rc = ensure_loaded(nl, b->mode, dig))) return rc;
             b->generated = true;
             b->gen_kernel[dig] = reinterpret_cast<const void*>(nl->gen[b->mode][dig].kernel);
+            b->cycle_kernel[dig] = reinterpret_cast<const void*>(nl->gen[b->mode][dig].cycle_kernel);
             // the input values of the current and the next cycle (generated
             // process functions read them instead of hashing every input)
             const size_t n_in = nl->nl.in_w.size();

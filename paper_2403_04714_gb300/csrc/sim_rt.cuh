@@ -264,23 +264,30 @@ namespace rtl {
 
 // Same cycle loop as the bytecode kernel.  LANE_INST (mode 2): every lane runs
 // its instance through the process function.  LANE_OP (mode 1): lane 0 runs
-// the process for one instance.
-template <int MODE, bool DIGEST>
+// the process for one instance.  VIEWS: launches of many cycles.
+template <int MODE, bool DIGEST, bool VIEWS>
 __device__ __forceinline__ void gen_cycles(const DevProg* __restrict__ P_dev, const DevState* __restrict__ S_dev,
                                            const LaunchArgs& A) {
     // The views in shared memory: the process functions read their base
     // pointers from them, and in global memory every barrier's acquire would
     // send those reads back to L2, in front of the first state loads
-    // (2k-op netlist x 1,000: 3.71 -> 3.36 us a cycle).
-    __shared__ DevProg P;
-    __shared__ DevState S;
-    for (uint32_t i = threadIdx.x; i < sizeof(DevProg) / 4; i += blockDim.x)
-        reinterpret_cast<uint32_t*>(&P)[i] = reinterpret_cast<const uint32_t*>(P_dev)[i];
-    for (uint32_t i = threadIdx.x; i < sizeof(DevState) / 4; i += blockDim.x)
-        reinterpret_cast<uint32_t*>(&S)[i] = reinterpret_cast<const uint32_t*>(S_dev)[i];
-    __syncthreads();
-    const DevProg* Pg = &P;
-    const DevState* Sg = &S;
+    // (2k-op netlist x 1,000: 3.71 -> 3.36 us a cycle).  A launch of one cycle
+    // has no such barrier, and the copy is a round trip in front of its only
+    // cycle (launches from graphs, 2k-op netlist x 700: 4.37 us a cycle with it,
+    // 3.92 without; 20k-op x 2,500 23.3, 21.4; 200k-op x 100 15.4, 14.9).
+    __shared__ DevProg P_sm;
+    __shared__ DevState S_sm;
+    if (VIEWS) {
+        for (uint32_t i = threadIdx.x; i < sizeof(DevProg) / 4; i += blockDim.x)
+            reinterpret_cast<uint32_t*>(&P_sm)[i] = reinterpret_cast<const uint32_t*>(P_dev)[i];
+        for (uint32_t i = threadIdx.x; i < sizeof(DevState) / 4; i += blockDim.x)
+            reinterpret_cast<uint32_t*>(&S_sm)[i] = reinterpret_cast<const uint32_t*>(S_dev)[i];
+        __syncthreads();
+    }
+    const DevProg* Pg = VIEWS ? &P_sm : P_dev;
+    const DevState* Sg = VIEWS ? &S_sm : S_dev;
+    const DevProg& P = *Pg;
+    const DevState& S = *Sg;
     const uint32_t lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const uint32_t tw = gridDim.x * A.warps_per_cta;
     const uint64_t t_base = A.t0_dev ? *A.t0_dev + A.t0 : A.t0;
@@ -358,15 +365,20 @@ __device__ __forceinline__ void gen_cycles(const DevProg* __restrict__ P_dev, co
 #define RTLSIM_GEN_MAX_THREADS 1024
 #endif
 
-// One kernel per generated module: rtl_gen_d1 (digests on) calls process
-// functions that carry the digest code, rtl_gen_d0 calls ones without it.
+// Two kernels per generated module: rtl_gen_d1 (digests on) calls process
+// functions that carry the digest code, rtl_gen_d0 calls ones without it;
+// rtl_cyc_d1 and rtl_cyc_d0 are the same for launches of one cycle.
 #define RTLSIM_GEN_KERNEL_NAME_false rtl_gen_d0
 #define RTLSIM_GEN_KERNEL_NAME_true rtl_gen_d1
+#define RTLSIM_CYC_KERNEL_NAME_false rtl_cyc_d0
+#define RTLSIM_CYC_KERNEL_NAME_true rtl_cyc_d1
 #define RTLSIM_GEN_CAT(a, b) a##b
-#define RTLSIM_GEN_KERNEL(MODE, DIGEST)                                                                       \
+#define RTLSIM_GEN_ENTRY(NAME, MODE, DIGEST, PERSISTENT)                                                      \
     extern "C" __global__ void __launch_bounds__(RTLSIM_GEN_MAX_THREADS)                                      \
-        RTLSIM_GEN_CAT(RTLSIM_GEN_KERNEL_NAME_, DIGEST)(const rtl::DevProg* P, const rtl::DevState* S,        \
-                                                        rtl::LaunchArgs A) {                                  \
-        rtl::gen_cycles<MODE, DIGEST>(P, S, A);                                                               \
+        NAME(const rtl::DevProg* P, const rtl::DevState* S, rtl::LaunchArgs A) {                              \
+        rtl::gen_cycles<MODE, DIGEST, PERSISTENT>(P, S, A);                                                   \
     }
+#define RTLSIM_GEN_KERNEL(MODE, DIGEST)                                                                       \
+    RTLSIM_GEN_ENTRY(RTLSIM_GEN_CAT(RTLSIM_GEN_KERNEL_NAME_, DIGEST), MODE, DIGEST, true)                     \
+    RTLSIM_GEN_ENTRY(RTLSIM_GEN_CAT(RTLSIM_CYC_KERNEL_NAME_, DIGEST), MODE, DIGEST, false)
 #endif
