@@ -32,10 +32,10 @@ struct GenModule {
     bool cached = false;
 };
 
-// Compile the units with NVRTC (relocatable cubins, in parallel) and link them
-// with nvJitLink (no GPU needed).  Linked cubins are cached on disk under
+// Compile the units of lane mapping `mode` with NVRTC (relocatable cubins, in
+// parallel) and link them with nvJitLink (no GPU needed).  Linked cubins are cached on disk under
 // `cache_dir` (empty: no cache) by a hash of the sources and options.
-int jit_compile(const std::vector<GenUnit>& units, const std::string& cache_dir, std::vector<char>& linked,
+int jit_compile(const std::vector<GenUnit>& units, int mode, const std::string& cache_dir, std::vector<char>& linked,
                 bool* cached, double* seconds, std::string& err);
 // Load a linked cubin on the current device and look up its kernel.
 int jit_load(const std::vector<char>& linked, bool digest, GenModule& out, std::string& err);

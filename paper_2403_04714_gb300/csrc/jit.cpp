@@ -60,21 +60,24 @@ void write_file(const std::string& path, const std::vector<char>& data) {
 // CTA per SM.  Measured on the 200k-op netlist with 4,096 instances (us per
 // simulated cycle, best CTA size): 48 registers 198, 56 204, 64 186, 72 197,
 // 80 203, 96 216.  At 64 the state's constant offsets (reg_pos) leave few
-// spills (27 local loads per task) and 32 warps share an SM.
-std::string max_registers() {
+// spills (27 local loads per task) and 32 warps share an SM.  With lane =
+// operation every address is computed, and 64 registers spill more than the
+// warps are worth (200k-op netlist, us a cycle at 64 and 80: one instance 21.1 and
+// 20.5, five 111.0 and 107.1, twenty 540 and 483).
+std::string max_registers(int mode) {
     const char* m = getenv("RTLSIM_GEN_MAXRREG");
-    return m ? m : "64";
+    return m ? m : mode == SIM_MODE_LANE_OP ? "80" : "64";
 }
 
 // The kernel entry's launch bound must leave every process function its
 // register cap: the largest CTA, in groups of 4 warps (one per SM
 // sub-partition), whose threads x cap fit the 65,536-register file.
-int max_threads() {
-    const int cap = std::max(16, std::min(255, atoi(max_registers().c_str())));
+int max_threads(int mode) {
+    const int cap = std::max(16, std::min(255, atoi(max_registers(mode).c_str())));
     return std::max(128, std::min(1024, 65536 / (cap * 128) * 128));
 }
 
-int compile_unit(const GenUnit& u, std::vector<char>& cubin, std::string& err) {
+int compile_unit(const GenUnit& u, int mode, std::vector<char>& cubin, std::string& err) {
     nvrtcProgram prog;
     const char* hdr[2] = {kEmbeddedAbiHeader, kEmbeddedRtHeader};
     const char* hdr_names[2] = {"abi_device.h", "sim_rt.cuh"};
@@ -84,9 +87,9 @@ int compile_unit(const GenUnit& u, std::vector<char>& cubin, std::string& err) {
     }
     std::string arch = std::string("--gpu-architecture=") + kArch;
     std::vector<const char*> opts = {arch.c_str(), "-rdc=true", "--std=c++17", "-default-device", "-w"};
-    std::string maxr = "--maxrregcount=" + max_registers();
+    std::string maxr = "--maxrregcount=" + max_registers(mode);
     opts.push_back(maxr.c_str());
-    std::string thr = "-DRTLSIM_GEN_MAX_THREADS=" + std::to_string(max_threads());
+    std::string thr = "-DRTLSIM_GEN_MAX_THREADS=" + std::to_string(max_threads(mode));
     opts.push_back(thr.c_str());
     nvrtcResult r = nvrtcCompileProgram(prog, int(opts.size()), opts.data());
     if (r != NVRTC_SUCCESS) {
@@ -139,12 +142,12 @@ int link_units(const std::vector<std::vector<char>>& cubins, const std::vector<G
 
 }  // namespace
 
-int jit_compile(const std::vector<GenUnit>& units, const std::string& cache_dir, std::vector<char>& linked,
+int jit_compile(const std::vector<GenUnit>& units, int mode, const std::string& cache_dir, std::vector<char>& linked,
                 bool* cached, double* seconds, std::string& err) {
     auto t0 = std::chrono::steady_clock::now();
     uint64_t h = 0xcbf29ce484222325ULL;
     h = fnv1a(h, kArch);
-    h = fnv1a(h, "maxrreg=" + max_registers() + " threads=" + std::to_string(max_threads()));
+    h = fnv1a(h, "maxrreg=" + max_registers(mode) + " threads=" + std::to_string(max_threads(mode)));
     h = fnv1a(h, kEmbeddedAbiHeader);
     h = fnv1a(h, kEmbeddedRtHeader);
     for (auto& u : units) h = fnv1a(fnv1a(h, u.name), u.source);
@@ -161,7 +164,7 @@ int jit_compile(const std::vector<GenUnit>& units, const std::string& cache_dir,
         std::vector<std::thread> th;
         for (unsigned k = 0; k < nt; k++)
             th.emplace_back([&] {
-                for (size_t i; (i = next.fetch_add(1)) < units.size();) rcs[i] = compile_unit(units[i], cubins[i], errs[i]);
+                for (size_t i; (i = next.fetch_add(1)) < units.size();) rcs[i] = compile_unit(units[i], mode, cubins[i], errs[i]);
             });
         for (auto& t : th) t.join();
         for (size_t i = 0; i < units.size(); i++)

@@ -540,7 +540,7 @@ int ensure_compiled(sim_netlist* h, int mode, bool digest) {
     }
     bool cached = false;
     double sec = 0;
-    rc = rtl::jit_compile(units, cache, h->gen_cubin[mode][digest], &cached, &sec, err);
+    rc = rtl::jit_compile(units, mode, cache, h->gen_cubin[mode][digest], &cached, &sec, err);
     if (rc) return set_err(rc, err);
     h->gen_seconds[mode][digest] = sec;
     h->gen_cached[mode][digest] = cached;
@@ -559,20 +559,25 @@ int ensure_loaded(sim_netlist* h, int mode, bool digest) {
 }
 
 // Warps per CTA and grid of generated code for b->n_tasks, on 1 / share of the
-// GPU.  Up to 1024 threads per CTA at 64 registers per thread.  Few tasks are
-// spread over the SMs in smaller CTAs (200k-op netlist, 304 tasks of 32
-// instances each: 24.3 us a cycle with 8 warps per CTA, 14.9 with 2; 64
-// instances: 18.2 with 8, 15.1 with 4); from 8 per SM on, 8 or more measured best.
+// GPU.  Up to 1024 threads per CTA at 64 registers per thread, 768 at 80 (lane =
+// operation).  Few tasks are spread over the SMs in smaller CTAs (200k-op
+// netlist, 304 tasks of 32 instances each: 24.3 us a cycle with 8 warps per CTA,
+// 14.9 with 2; 64 instances: 18.2 with 8, 15.1 with 4); from 8 per SM on, 8 or
+// more measured best.
 int plan_grid_gen(sim_batch* b, uint32_t share) {
     g_counts[SIM_COUNT_PLANS]++;
     const int sms = sm_count();
     const int spread = int(std::min<uint32_t>(8, std::max<uint32_t>(2, (b->n_tasks + sms - 1) / sms)));
     b->warps = std::min(32, b->cfg.warps_per_cta ? int(b->cfg.warps_per_cta) : spread);
-    b->threads = b->warps * 32;
     int occ = 0;
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, b->gen_kernel[b->cfg.digest_capacity > 0],
-                                                           b->threads, 0));
-    if (occ < 1) return set_err(SIM_ERR_CAPACITY, "generated kernel does not fit on an SM");
+    // (a CTA of more warps than its registers leave room for is halved)
+    for (;; b->warps /= 2) {
+        b->threads = b->warps * 32;
+        CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, b->gen_kernel[b->cfg.digest_capacity > 0],
+                                                               b->threads, 0));
+        if (occ > 0) break;
+        if (b->warps == 1) return set_err(SIM_ERR_CAPACITY, "generated kernel does not fit on an SM");
+    }
     b->max_grid = occ * sms;
     const int need = int((b->n_tasks + b->warps - 1) / b->warps);
     b->grid = std::max(1, std::min(need, std::max(1, b->max_grid / int(std::max(1u, share)))));

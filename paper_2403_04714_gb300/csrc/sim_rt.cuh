@@ -359,8 +359,8 @@ __device__ __forceinline__ void gen_cycles(const DevProg* __restrict__ P_dev, co
 
 }  // namespace rtl
 
-// Threads per CTA the generated kernels are compiled for: 1024 at the default
-// 64-register cap; a higher cap (RTLSIM_GEN_MAXRREG) compiles for fewer.
+// Threads per CTA the generated kernels are compiled for: 1024 at a cap of 64
+// registers; a higher one (lane = operation, RTLSIM_GEN_MAXRREG) compiles for fewer.
 #ifndef RTLSIM_GEN_MAX_THREADS
 #define RTLSIM_GEN_MAX_THREADS 1024
 #endif
