@@ -26,8 +26,8 @@ struct LanePlan {
     size_t smem = 0;
 };
 
-// The CTA size and grid with the fewest rounds of tasks, then the fewest
-// warps.  slots(i): value slots of the i-th process, descending.  occ(threads,
+// Persistent launches: the CTA size and grid with the fewest rounds of tasks,
+// then the fewest warps.  slots(i): value slots of the i-th process, descending.  occ(threads,
 // smem, &ctas): CTAs that fit on an SM, or an error code, which ends the search.
 template <class Slots, class Occ>
 int plan_lane(const LanePlanInput& in, Slots&& slots, Occ&& occ, LanePlan& best) {
@@ -39,6 +39,33 @@ int plan_lane(const LanePlanInput& in, Slots&& slots, Occ&& occ, LanePlan& best)
         return size_t(words) * 8;
     };
     best = LanePlan();
+    if (in.per_cycle && !in.warps) {
+        // The CTAs of a launch of one cycle follow one another on an SM as they
+        // finish, and a large one leaves it to its last warps.  So CTAs of four
+        // warps (fewer where there are not four tasks for every SM), or of as many
+        // as make fewer waves of resident warps.  Chosen as for persistent
+        // launches, us a cycle: 2k-op netlist x 2,500 19 warps 32.2, 4 warps 18.1;
+        // 20k-op x 2,500 32 warps 298, 4 warps 219; 200k-op x 2,500 4 warps 1,840,
+        // 20 warps 1,647.
+        const int base = int(std::min<uint64_t>(4, std::max<uint64_t>(1, (n_tasks + in.sms - 1) / in.sms)));
+        for (int i = 0; i <= 32; i++) {
+            const int w = i ? i : base;
+            const uint32_t need = (n_tasks + w - 1) / w;
+            const size_t smem = area_bytes(w, need);
+            if (smem > in.smem_limit) continue;
+            int ctas = 0;
+            if (int rc = occ(w * 32, smem, &ctas)) return rc;
+            const uint64_t warps = uint64_t(ctas) * w * in.sms;
+            if (!warps || (n_tasks + warps - 1) / warps >= best.rounds) continue;
+            best.rounds = (n_tasks + warps - 1) / warps;
+            best.warps = w;
+            best.smem = smem;
+            best.max_grid = ctas * in.sms;
+            best.grid = int(std::min(need, std::max(1u, uint32_t(best.max_grid) / share)));
+        }
+        if (best.warps) best.rounds = (n_tasks + uint64_t(best.grid) * best.warps - 1) / (uint64_t(best.grid) * best.warps);
+        return 0;
+    }
     int lo = in.warps ? int(std::min(32u, in.warps)) : 1, hi = in.warps ? lo : 32;
     // (a configured CTA size that does not fit is halved until it does)
     for (; best.rounds == ~0ull && lo >= 1; lo = lo / 2, hi = lo) {
