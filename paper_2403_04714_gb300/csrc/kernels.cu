@@ -615,7 +615,9 @@ __device__ __forceinline__ void lane_inst_packed(const DevProg& P, const DevStat
             task_lane_inst<DIGEST>(P, S, proc(task), task % G, t, c > 0 || A.pending_first, sl, block, lane);
         if (A.grid_sync) {
             const bool skip = (int32_t)blockIdx.x == A.skip_cta && c == 0;
-            if (!grid_barrier(S.bar, gen, A.timeout_ns, S.err, skip, rec ? rec + 1 : nullptr)) return;
+            // (its processes take microseconds: the polls of a wide grid do not tell,
+            // and asking for its width made the task loop 0.5 % slower)
+            if (!grid_barrier<false>(S.bar, gen, A.timeout_ns, S.err, skip, rec ? rec + 1 : nullptr)) return;
         }
     }
     if (A.grid_sync && A.n > 0)
@@ -690,7 +692,7 @@ __global__ void __launch_bounds__(1024) k_cycles(DevProg P, DevState S, LaunchAr
         }
         if (A.grid_sync) {
             bool skip = (int32_t)blockIdx.x == A.skip_cta && c == 0;
-            if (!grid_barrier(S.bar, gen, A.timeout_ns, S.err, skip, rec ? rec + 1 : nullptr)) return;
+            if (!grid_barrier<MODE != SIM_MODE_LANE_INST>(S.bar, gen, A.timeout_ns, S.err, skip, rec ? rec + 1 : nullptr)) return;
         }
     }
     if (A.grid_sync && A.n > 0)

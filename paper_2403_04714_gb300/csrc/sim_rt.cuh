@@ -62,6 +62,8 @@ constexpr uint32_t kQuickPollCtas = 608;     // four per SM
 // an error, the CTA records SIM_ERR_TIMEOUT (first error wins) and returns
 // false.  With `rec` set, thread 0 stores the time the whole CTA arrived
 // (rec[0]) and the time the barrier released it (rec[1]), from %globaltimer.
+// WIDE: the grid may have more than kQuickPollCtas CTAs.
+template <bool WIDE = true>
 static __device__ bool grid_barrier(uint32_t* bar, uint32_t& gen, uint64_t timeout_ns, int32_t* err, bool skip,
                                     uint64_t* rec = nullptr) {
     __shared__ int s_ok;
@@ -72,7 +74,7 @@ static __device__ bool grid_barrier(uint32_t* bar, uint32_t& gen, uint64_t timeo
         unsigned long long* count = reinterpret_cast<unsigned long long*>(bar);
         const unsigned long long target = (unsigned long long)(gen + 1) * gridDim.x;
         if (!skip) red_release_add(count, 1ull);
-        const uint32_t quick = gridDim.x <= kQuickPollCtas ? 15u : 0u;
+        const uint32_t quick = !WIDE || gridDim.x <= kQuickPollCtas ? 15u : 0u;
         uint64_t start = 0;
         for (uint32_t polls = 1; ld_acquire_u64(count) < target; polls++) {
             if (polls & quick) continue;
