@@ -975,9 +975,13 @@ int init_state(sim_batch* b) {
             if (!bytes) return SIM_OK;
             char* d = static_cast<char*>(dst);
             const size_t first = std::min(tiles, std::max<size_t>(1, (size_t(1) << 20) / bytes));
-            host[k].resize(bytes * first);
-            for (size_t t = 0; t < first; t++) memcpy(host[k].data() + t * bytes, tile, bytes);
-            CUDA_TRY(cudaMemcpyAsync(d, host[k].data(), bytes * first, cudaMemcpyHostToDevice, st));
+            const void* src = tile;
+            if (first > 1) {
+                host[k].resize(bytes * first);
+                for (size_t t = 0; t < first; t++) memcpy(host[k].data() + t * bytes, tile, bytes);
+                src = host[k].data();
+            }
+            CUDA_TRY(cudaMemcpyAsync(d, src, bytes * first, cudaMemcpyHostToDevice, st));
             for (size_t done = bytes * first, n; done < bytes * tiles; done += n) {
                 n = std::min(done, bytes * tiles - done);
                 CUDA_TRY(cudaMemcpyAsync(d + done, d, n, cudaMemcpyDeviceToDevice, st));
