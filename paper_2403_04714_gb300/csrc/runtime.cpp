@@ -567,7 +567,14 @@ int ensure_loaded(sim_netlist* h, int mode, bool digest) {
 int plan_grid_gen(sim_batch* b, uint32_t share) {
     g_counts[SIM_COUNT_PLANS]++;
     const int sms = sm_count();
-    const int spread = int(std::min<uint32_t>(8, std::max<uint32_t>(2, (b->n_tasks + sms - 1) / sms)));
+    // (launches of one cycle with processes of less than 32 operators on average
+    // are over before the spread is worth its CTAs: 2k-op netlist, mean 23, x 32
+    // from graphs 3.60 us a cycle with 2 warps per CTA, 3.44 with 8, x 64 3.84 and
+    // 3.55; 5k-op netlist, mean 38, x 32 3.69 and 4.19)
+    const sim_netlist_info& I = b->nl->info;
+    const bool brief = (b->kernel == SIM_KERNEL_PER_CYCLE || b->kernel == SIM_KERNEL_PER_CYCLE_GRAPH) &&
+                       I.process_cost_sum < 32ull * I.n_processes;
+    const int spread = brief ? 8 : int(std::min<uint32_t>(8, std::max<uint32_t>(2, (b->n_tasks + sms - 1) / sms)));
     b->warps = std::min(32, b->cfg.warps_per_cta ? int(b->cfg.warps_per_cta) : spread);
     int occ = 0;
     // (a CTA of more warps than its registers leave room for is halved)

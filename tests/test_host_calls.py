@@ -103,6 +103,16 @@ for warps in (1, 2, 3, 4, 6, 8):
         rounds = -(-need // most)
         assert i["ctas"] == (-(-need // rounds) if warps <= 4 else min(need, most)), (warps, n, i)
         b.close()
+
+# launches of one cycle: few tasks are spread over the SMs unless they are brief
+def warps(text, **cfg):
+    b = sim.Batch(sim.Netlist(text, mode="lane_inst", lowering="generated", **cfg), 32)
+    return b.launch_info()["warps_per_cta"]
+
+longer = netgen.gen_flat(21, 5000, 400, 20, 9).to_text()
+assert warps(text) == 2 and warps(longer) == 2
+assert warps(text, kernel="graph") == 8 and warps(text, kernel="per_cycle") == 8
+assert warps(longer, kernel="graph") == 2 and warps(text, kernel="persistent_graph") == 2
 print("done")
 """
 
