@@ -67,7 +67,8 @@ enum { SIM_SIG_INPUT = 0, SIM_SIG_REG = 1 };
  *   LANE_OP:   one warp runs one process of one instance; its 32 lanes run
  *              independent nodes of the same schedule step (single instance).
  *   LANE_INST: one warp runs one process for 32 instances, lane = instance,
- *              with instance-minor state (batched stimulus instances).
+ *              with the registers in tiles of 32 instances (batched stimulus
+ *              instances).
  *   AUTO:      LANE_INST when n_inst >= 32, else LANE_OP. */
 enum { SIM_MODE_AUTO = 0, SIM_MODE_LANE_OP = 1, SIM_MODE_LANE_INST = 2 };
 

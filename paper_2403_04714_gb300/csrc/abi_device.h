@@ -89,8 +89,6 @@ constexpr uint32_t kOpMaskShift = 25;         // 64 - width (64: mask 0)
 // Constant table (64-bit words): 0, ~0, the powers of two, then 3, 5, 6, 7, 9, ... 63.
 constexpr uint32_t kTabZero = 0, kTabOnes = 1, kTabPow2 = 2, kTabInts = 66, kTabWords = 124;
 
-
-
 // Program tables of one lowered netlist (device pointers).
 struct DevProg {
     const DIns* s_ins;          // LANE_OP bundles (32 instructions per row)
@@ -113,8 +111,8 @@ struct DevProg {
     const uint8_t* in_w;
     const uint8_t* reg_cls;
     const uint32_t* reg_idx;
-    // cluster exchange (null unless the netlist was lowered for clusters)
     const uint32_t* proc_order; // processes by descending cost (generated code, process-major order)
+    // cluster exchange (null unless the netlist was lowered for clusters)
     const uint32_t* warp_proc;  // process of each warp of the grid, kNoProc if idle
     const uint32_t* mir_off;    // per CTA: first mirror entry (grid+1 offsets)
     const uint32_t* mir_reg;    // register held by each mirror entry

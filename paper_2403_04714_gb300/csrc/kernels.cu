@@ -374,18 +374,6 @@ __device__ void task_lane_op(const DevProg& P, const DevState& S, uint32_t p, ui
     finish_lane_op<DIGEST>(S, p, inst, t, col, lane, dacc);
 }
 
-// One operator of a shared-memory program (abi_device.h has the formula).
-// Bound by the issue of its dependent instructions, one warp per scheduler
-// most of the time and about five lanes with an operator each; so it forms no
-// candidate that a constant operand can switch off instead, and the next
-// step's operators are loaded while this one's are evaluated.  200k-op netlist,
-// one instance, against a select tree over every operator's result: 12.3 ->
-// 9.0 us a cycle on the grid barrier (63 steps; 11.0 without the early load),
-// 10.5 -> 9.1 with operator pairs in 2-CTA clusters (38 steps), 499k-op mesh
-// 15.9 -> 10.5, 2k-op netlist in one cluster 3.8 -> 3.2.  Measured slower:
-// A == X and A < c from the selected operand (2 %), the result of a compare
-// selected in 64 bits (2-4 %), fields read as 16-bit words (3-5 %), the fields
-// taken apart before the warp barrier (no change), the mask as two shifts (5 %).
 // All bits of the result: the sign bit of byte BYTE of v.
 template <int BYTE>
 __device__ __forceinline__ uint64_t byte_sign(uint32_t v) {
@@ -402,6 +390,18 @@ __device__ __forceinline__ OpFields op_fields(uint4 o) {
     return {o.y & 0xffffu, o.y >> 16, o.z & 0xffffu, o.z >> 16, o.x >> 16, o.x, o.w};
 }
 
+// One operator of a shared-memory program (abi_device.h has the formula).
+// Bound by the issue of its dependent instructions, one warp per scheduler
+// most of the time and about five lanes with an operator each; so it forms no
+// candidate that a constant operand can switch off instead, and the next
+// step's operators are loaded while this one's are evaluated.  200k-op netlist,
+// one instance, against a select tree over every operator's result: 12.3 ->
+// 9.0 us a cycle on the grid barrier (63 steps; 11.0 without the early load),
+// 10.5 -> 9.1 with operator pairs in 2-CTA clusters (38 steps), 499k-op mesh
+// 15.9 -> 10.5, 2k-op netlist in one cluster 3.8 -> 3.2.  Measured slower:
+// A == X and A < c from the selected operand (2 %), the result of a compare
+// selected in 64 bits (2-4 %), fields read as 16-bit words (3-5 %), the fields
+// taken apart before the warp barrier (no change), the mask as two shifts (5 %).
 __device__ __forceinline__ uint64_t eval_op(uint32_t w0, uint32_t bits, uint64_t a, uint64_t m, uint64_t x, uint64_t d, bool inv) {
     const uint64_t k_and = byte_sign<1>(bits), k_orx = byte_sign<2>(bits);
     const bool P = (d != 0) != inv;
@@ -683,11 +683,12 @@ __global__ void __launch_bounds__(1024) k_cycles(DevProg P, DevState S, LaunchAr
             for (uint32_t task = warp; task < A.n_tasks; task += tw) {
                 // process-major order: neighbouring warps run the same process
                 // for different instance groups (its code and constants stay hot)
-            uint32_t p, g;
-            task_coords(A, P.n_proc, task, p, g);
-                if (MODE == SIM_MODE_LANE_INST) task_lane_inst<DIGEST>(P, S, p, g, t, pending, sl,
-                                                                              reinterpret_cast<uint4*>(sl + A.slot_words - kBlockWords), lane);
-                else task_lane_op<DIGEST>(P, S, p, g, t, pending, sl, lane);
+                uint32_t p, g;
+                task_coords(A, P.n_proc, task, p, g);
+                if (MODE == SIM_MODE_LANE_INST)
+                    task_lane_inst<DIGEST>(P, S, p, g, t, pending, sl, reinterpret_cast<uint4*>(sl + A.slot_words - kBlockWords), lane);
+                else
+                    task_lane_op<DIGEST>(P, S, p, g, t, pending, sl, lane);
             }
         }
         if (A.grid_sync) {

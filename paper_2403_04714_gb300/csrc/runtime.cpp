@@ -602,7 +602,7 @@ int plan_grid_gen(sim_batch* b, uint32_t share) {
     return SIM_OK;
 }
 
-// Launch plan for generated code: no shared memory, occupancy from registers.
+// Launch plan for generated code: no dynamic shared memory, occupancy from registers.
 int plan_launch_gen(sim_batch* b) {
     const uint32_t n_proc = uint32_t(b->nl->part.procs.size());
     b->n_tasks = b->mode == SIM_MODE_LANE_INST ? n_proc * (b->I / 32) : n_proc * b->I;
