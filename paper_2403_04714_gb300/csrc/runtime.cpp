@@ -1751,12 +1751,15 @@ int sim_save(sim_batch* b, void** blob, size_t* len) {
     BlobHeader h{kMagic, 1, b->nl->nl.reg_w.size(), b->nl->mem_word_off.back(), S.I, uint64_t(b->mode), b->cycle, b->nl->nl.in_w.size()};
     memcpy(p, &h, sizeof h);
     char* q = p + sizeof h;
+    // one wait for all of them, which makes up for the kernel above
     auto d2h = [&](const void* src, size_t n) {
-        if (n && b->d2h(q, src, n) != SIM_OK) return false;
+        if (n && cudaMemcpyAsync(q, src, n, cudaMemcpyDeviceToHost, b->stream) != cudaSuccess) return false;
         q += n;
         return true;
     };
-    if (!d2h(S.bits[par], nb) || !d2h(S.w32[par], n32) || !d2h(S.w64[par], n64) || !d2h(S.mem, nm) || !d2h(S.mem_dig, nmd)) {
+    const bool queued = d2h(S.bits[par], nb) && d2h(S.w32[par], n32) && d2h(S.w64[par], n64) && d2h(S.mem, nm) && d2h(S.mem_dig, nmd);
+    if (cudaStreamSynchronize(b->stream) != cudaSuccess || !queued) {
+        (void)cudaGetLastError();
         free(p);
         return set_err(SIM_ERR_CUDA, "checkpoint copy failed");
     }
@@ -1790,27 +1793,29 @@ int sim_restore(sim_batch* b, const void* blob, size_t len) {
     const bool tiled = S.pack == 32;
     const uint32_t par = uint32_t(h.cycle & 1) ^ (tiled ? 1u : 0u);
     const char* q = static_cast<const char*>(blob) + sizeof h;
+    // one wait for all of them, which makes up for the kernel below
     auto h2d = [&](void* dst, size_t n) {
-        if (n && b->h2d(dst, q, n) != SIM_OK) return false;
+        if (n && cudaMemcpyAsync(dst, q, n, cudaMemcpyHostToDevice, b->stream) != cudaSuccess) return false;
         q += n;
         return true;
     };
-    if (!h2d(S.bits[par], nb) || !h2d(S.w32[par], n32) || !h2d(S.w64[par], n64) || !h2d(S.mem, nm) || !h2d(S.mem_dig, nmd))
-        return set_err(SIM_ERR_CUDA, "restore copy failed");
-    if (tiled) {
+    bool queued = h2d(S.bits[par], nb) && h2d(S.w32[par], n32) && h2d(S.w64[par], n64) && h2d(S.mem, nm) && h2d(S.mem_dig, nmd);
+    if (queued && tiled) {
         OnDevice on(b->device);
-        CUDA_TRY(launch_retile(b->stream, S, par ^ 1u, true));
+        queued = launch_retile(b->stream, S, par ^ 1u, true) == cudaSuccess;
     }
-    if (nh) {
+    if (queued && nh) {
         memcpy(b->h_hold_val.data(), q, nh * 8);
-        q += nh * 8;
-        memcpy(b->h_hold_flag.data(), q, nh);
-        if ((rc = b->h2d(b->hold_val.p, b->h_hold_val.data(), nh * 8))) return rc;
-        if ((rc = b->h2d(b->hold_flag.p, b->h_hold_flag.data(), nh))) return rc;
+        memcpy(b->h_hold_flag.data(), q + nh * 8, nh);
+        queued = h2d(b->hold_val.p, nh * 8) && h2d(b->hold_flag.p, nh);
         S.any_hold = std::any_of(b->h_hold_flag.begin(), b->h_hold_flag.end(), [](uint8_t f) { return f != 0; });
     }
-    for (int k = 0; k < 2; k++)
-        if (b->rec[k].n) CUDA_TRY(cudaMemsetAsync(b->rec[k].p, 0, b->rec[k].n, b->stream));
+    for (int k = 0; k < 2 && queued; k++)
+        if (b->rec[k].n) queued = cudaMemsetAsync(b->rec[k].p, 0, b->rec[k].n, b->stream) == cudaSuccess;
+    if (cudaStreamSynchronize(b->stream) != cudaSuccess || !queued) {
+        (void)cudaGetLastError();
+        return set_err(SIM_ERR_CUDA, "restore copy failed");
+    }
     b->cycle = h.cycle;
     b->failed = false;
     b->fail_reason.clear();
