@@ -1,6 +1,7 @@
 // runtime.cpp -- C ABI of the simulator (include/sim.h): netlist handles,
 // batches of instances in device memory, stepping, peek/poke, digests.
 #include <cuda_runtime.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <atomic>
@@ -1735,7 +1736,9 @@ int sim_save(sim_batch* b, void** blob, size_t* len) {
     if (!p) return set_err(SIM_ERR_OOM, "host allocation failed");
     // touch the pages while a step may still run: a copy into pages that are
     // not mapped yet faults on the device for each (21 MB: 21 ms instead of 1.6)
-    for (size_t i = 0; i < total; i += 4096) p[i] = 0;
+    const size_t page = size_t(std::max(4096l, sysconf(_SC_PAGESIZE)));     // 64 KB on GB300's host
+    for (size_t i = 0; i < total; i += page) p[i] = 0;
+    p[total - 1] = 0;
     // registers in [register][instance] order whatever the kernels' layout
     uint32_t par = uint32_t(b->cycle & 1);
     int rc = sim_sync(b);
