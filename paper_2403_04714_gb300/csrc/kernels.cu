@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(1024) k_cycles_cl(DevProg P, DevState S, Launc
         } else if (A.one_cluster)
             ok = cluster_barrier(cbar, c, A.cluster, A.timeout_ns, S.err, skip, rec ? rec + 1 : nullptr);
         else
-            ok = grid_barrier(S.bar, gen, A.timeout_ns, S.err, skip, rec ? rec + 1 : nullptr);
+            ok = grid_barrier<false>(S.bar, gen, A.timeout_ns, S.err, skip, rec ? rec + 1 : nullptr);
     }
     cluster_sync_all();   // no CTA exits while a peer may still write into its shared memory
     if (ok && A.n > 0)

@@ -74,10 +74,9 @@ static __device__ bool grid_barrier(uint32_t* bar, uint32_t& gen, uint64_t timeo
         unsigned long long* count = reinterpret_cast<unsigned long long*>(bar);
         const unsigned long long target = (unsigned long long)(gen + 1) * gridDim.x;
         if (!skip) red_release_add(count, 1ull);
-        const uint32_t quick = !WIDE || gridDim.x <= kQuickPollCtas ? 15u : 0u;
         uint64_t start = 0;
         for (uint32_t polls = 1; ld_acquire_u64(count) < target; polls++) {
-            if (polls & quick) continue;
+            if ((polls & 15u) && !(WIDE && gridDim.x > kQuickPollCtas)) continue;
             const uint64_t now = globaltimer_ns();
             if (!start) start = now;
             if (ld_volatile(err) != 0) { ok = 0; break; }
